@@ -467,6 +467,7 @@ std::vector<Op> merge_tile_diagonals(std::vector<Op> ops, int max_k, double swee
             if (r != cd(1.0)) nt.push_back({qa, qh, r});
         }
         // the block with this op: qubits high-to-low, entries, terms
+        constexpr int kMaxDiag = 8;  // operands of an op, and the widest block
         auto extend = [&](std::vector<int> &nQ, std::vector<cd> &nD, std::vector<HiTerm> &nterms) {
             const bool fresh = members.empty();
             nQ = fresh ? lq : Q;
@@ -476,18 +477,25 @@ std::vector<Op> merge_tile_diagonals(std::vector<Op> ops, int max_k, double swee
             std::sort(nQ.begin(), nQ.end(), [](int a, int b) { return a > b; });
             const int K = (int)nQ.size();
             const int kl = (int)lq.size();
+            if (K > kMaxDiag) return;  // does not fit (checked by its qubits)
             nD.assign((size_t)1 << K, 1.0);
-            for (size_t x = 0; x < nD.size(); x++) {
-                auto bit_of = [&](int q) {
-                    for (int t = 0; t < K; t++)
-                        if (nQ[t] == q) return (int)((x >> (K - 1 - t)) & 1);
-                    return 0;
-                };
-                size_t xo = 0;  // index into the old block
-                for (size_t t = 0; t < Q.size(); t++) xo |= (size_t)bit_of(Q[t]) << (Q.size() - 1 - t);
-                size_t xm = 0;  // index into the op's local diagonal
-                for (int j = 0; j < kl; j++) xm |= (size_t)bit_of(lq[j]) << (kl - 1 - j);
-                nD[x] = (fresh ? cd(1.0) : D[xo]) * dl[xm];
+            // index into the old block (low half) and into the op's local diagonal (high half)
+            // of every entry, from its lowest set bit and the entry without it
+            uint32_t bit_index[kMaxDiag], index[1 << kMaxDiag];
+            for (int b = 0; b < K; b++) {
+                const int q = nQ[(size_t)(K - 1 - b)];
+                uint32_t w = 0;
+                for (size_t t = 0; t < Q.size(); t++)
+                    if (Q[t] == q) w |= 1u << (Q.size() - 1 - t);
+                for (int j = 0; j < kl; j++)
+                    if (lq[(size_t)j] == q) w |= 1u << (16 + kl - 1 - j);
+                bit_index[b] = w;
+            }
+            index[0] = 0;
+            for (uint32_t x = 0; x < (1u << K); x++) {
+                if (x) index[x] = index[x & (x - 1)] | bit_index[__builtin_ctz(x)];
+                const cd o = fresh ? cd(1.0) : D[index[x] & 0xFFFFu], m = dl[index[x] >> 16];
+                nD[x] = cd(o.real() * m.real() - o.imag() * m.imag(), o.real() * m.imag() + o.imag() * m.real());
             }
             nterms = fresh ? nt : terms;
             if (!fresh) nterms.insert(nterms.end(), nt.begin(), nt.end());
@@ -496,8 +504,9 @@ std::vector<Op> merge_tile_diagonals(std::vector<Op> ops, int max_k, double swee
         // with terms (so that table and terms fit one op's reals, and every table bit
         // with terms has a factor slot)
         auto fits = [&](const std::vector<int> &q, const std::vector<cd> &d, const std::vector<HiTerm> &tt) {
+            if ((int)q.size() > std::min(max_k, kMaxDiag)) return false;
             const int table_bits = (int)q.size() - controls(q, d, tt);
-            return (int)q.size() <= max_k && table_bits <= (tt.empty() ? max_k : max_k - 1) &&
+            return table_bits <= (tt.empty() ? max_k : max_k - 1) &&
                    tt.size() <= (size_t)kMaxHiTerms;
         };
         extend(nQ, nD, nterms);

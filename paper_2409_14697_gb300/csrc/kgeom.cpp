@@ -414,11 +414,12 @@ std::vector<KOp> build_register_phases(const std::vector<Op> &ops, const int *po
     // diagonal ops commute with one another: one left out only blocks later non-diagonal ops
     std::vector<char> diag(N);
     for (size_t i = 0; i < N; i++) diag[i] = op_is_diagonal(ops[i]);
-    auto trial = [&](size_t first, uint32_t allowed, std::vector<int> &taken) {
+    std::vector<int> open(N);  // ops not in a phase yet
+    for (size_t i = 0; i < N; i++) open[i] = (int)i;
+    auto trial = [&](uint32_t allowed, std::vector<int> &taken) {
         uint32_t R = 0, blocked = 0, blocked_diag = 0;
         taken.clear();
-        for (size_t i = first; i < N; i++) {
-            if (done[i]) continue;
+        for (int i : open) {
             const uint32_t tm = touch[i];
             const uint32_t blk = diag[i] ? blocked : (blocked | blocked_diag);
             bool take = ok[i] && !(tm & blk) && (int)taken.size() < kRpMaxMembers;
@@ -427,7 +428,7 @@ std::vector<KOp> build_register_phases(const std::vector<Op> &ops, const int *po
                 take = (need & ~allowed) == 0 && __builtin_popcount(R | need) <= kRpBits;
                 if (take) R |= need;
             }
-            if (take) taken.push_back((int)i);
+            if (take) taken.push_back(i);
             else if (diag[i]) blocked_diag |= tm;
             else blocked |= tm;
             if ((blocked & all) == all) break;
@@ -436,11 +437,11 @@ std::vector<KOp> build_register_phases(const std::vector<Op> &ops, const int *po
     };
     std::vector<KOp> out;
     int phases = 0;
-    size_t first = 0;
     std::vector<int> best, cand;
     while (true) {
-        while (first < N && done[first]) first++;
-        if (first >= N) break;
+        open.erase(std::remove_if(open.begin(), open.end(), [&](int i) { return done[i] != 0; }), open.end());
+        if (open.empty()) break;
+        const int first = open.front();
         if (!ok[first]) {
             out.push_back(make_tile_kop(ops[first], pos, mats));
             done[first] = 1;
@@ -448,9 +449,9 @@ std::vector<KOp> build_register_phases(const std::vector<Op> &ops, const int *po
         }
         // candidates: unrestricted, and register positions within each window of kRpBits
         // consecutive positions; keep the one that takes most ops
-        uint32_t R = trial(first, all, best);
+        uint32_t R = trial(all, best);
         for (int w = 0; w + kRpBits <= m; w++) {
-            const uint32_t Rw = trial(first, ((1u << kRpBits) - 1u) << w, cand);
+            const uint32_t Rw = trial(((1u << kRpBits) - 1u) << w, cand);
             if (cand.size() > best.size()) {
                 best.swap(cand);
                 R = Rw;

@@ -51,10 +51,9 @@ bool nonzero_entries(const cd (&d)[4], bool one_qubit) {
     return true;
 }
 
-cd ipow(cd z, int k) {
-    cd r = 1.0;
-    for (int i = 0; i < k; i++) r *= z;
-    return r;
+// The plain product (std::complex's operator also looks for infinities and NaN).
+cd mul(cd a, cd b) {
+    return cd(a.real() * b.real() - a.imag() * b.imag(), a.real() * b.imag() + a.imag() * b.real());
 }
 
 // std::complex has no ordering; key factors by their bit patterns.
@@ -151,15 +150,23 @@ std::shared_ptr<const PhaseFn> build_phasefn(const std::vector<Op> &ops, size_t 
         size *= (size_t)(g.max_count + 1);
         if (size > (size_t)kPfMaxTable) return nullptr;
     }
-    pf->table.assign(size, C);
-    for (size_t idx = 0; idx < size; idx++) {
-        size_t rest = idx;
-        for (const PfGroup &g : groups) {
-            const int c = (int)(rest % (size_t)(g.max_count + 1));
-            rest /= (size_t)(g.max_count + 1);
-            pf->table[idx] *= ipow(g.value, c);
-            if (g.kind == PF_WEIGHT && g.clique != cd(1.0)) pf->table[idx] *= ipow(g.clique, c * (c - 1) / 2);
-        }
+    // the table group by group: entry = the entry of the groups before it times value^count (and
+    // the clique's factor), counts of the first group varying fastest
+    pf->table.reserve(size);
+    pf->table.assign(1, C);
+    for (const PfGroup &g : groups) {
+        const size_t before = pf->table.size();
+        const bool clique = g.kind == PF_WEIGHT && g.clique != cd(1.0);
+        std::vector<cd> pw(1, 1.0), pc(1, 1.0);  // powers by repeated multiplication
+        for (int c = 1; c <= g.max_count; c++) pw.push_back(mul(pw.back(), g.value));
+        for (int e = 1; clique && e <= g.max_count * (g.max_count - 1) / 2; e++) pc.push_back(mul(pc.back(), g.clique));
+        pf->table.resize(before * (size_t)(g.max_count + 1));
+        for (int c = g.max_count; c >= 0; c--)
+            for (size_t i = 0; i < before; i++) {
+                cd z = mul(pf->table[i], pw[(size_t)c]);
+                if (clique) z = mul(z, pc[(size_t)(c * (c - 1) / 2)]);
+                pf->table[(size_t)c * before + i] = z;
+            }
     }
     pf->groups = std::move(groups);
     return pf;

@@ -139,10 +139,12 @@ struct Trial {
     bool stream = false;
 };
 
-// What the pass builder asks of each op, computed once per plan (a plan tries many passes).
+// What the pass builder asks of each op, computed once per plan (a plan tries many passes);
+// the ops of earlier passes leave the list.
 struct OpInfo {
     uint64_t qm;   // qubits
     uint64_t hi;   // qubits that may be its only local one (pp.hi_diag)
+    int index;
     bool diag;
     bool chunk;
 };
@@ -150,6 +152,7 @@ struct OpInfo {
 std::vector<OpInfo> op_info(const std::vector<Op> &ops, const PlanParams &pp) {
     std::vector<OpInfo> info(ops.size());
     for (size_t i = 0; i < ops.size(); i++) {
+        info[i].index = (int)i;
         info[i].qm = ops[i].qmask();
         info[i].diag = op_is_diagonal(ops[i]);
         info[i].chunk = chunkable(ops[i], pp);
@@ -158,32 +161,31 @@ std::vector<OpInfo> op_info(const std::vector<Op> &ops, const PlanParams &pp) {
     return info;
 }
 
-Trial greedy_pass(const std::vector<OpInfo> &ops, const std::vector<char> &done, size_t first, int n,
-                  const PlanParams &pp, uint64_t allowed) {
+void greedy_pass(const std::vector<OpInfo> &ops, int n, const PlanParams &pp, uint64_t allowed, Trial &tr) {
     const uint64_t all = (n >= 64) ? ~0ull : ((1ull << n) - 1ull);
     const uint64_t low = (1ull << pp.c) - 1ull;
-    Trial tr;
+    tr.ops.clear();
+    tr.stream = false;
     // qubits of ops left for a later pass: a non-diagonal op left behind blocks every later
     // op on its qubits; a diagonal one only blocks later non-diagonal ops (diagonal gates
     // commute with one another, so they may pass it)
     uint64_t L = low, blocked = 0, blocked_diag = 0;
-    for (size_t i = first; i < ops.size(); i++) {
-        if (done[i]) continue;
-        const OpInfo &op = ops[i];
+    for (const OpInfo &op : ops) {
+        const int i = op.index;
         const uint64_t qm = op.qm;
         const bool diag = op.diag;
         const uint64_t blk = diag ? blocked : (blocked | blocked_diag);
         if (!op.chunk) {
             if (tr.ops.empty() && !(qm & (blocked | blocked_diag))) {
                 tr.stream = true;
-                tr.ops.push_back((int)i);
+                tr.ops.push_back(i);
             }
             break;  // a non-chunkable op is a barrier for this pass
         }
         bool take = false;
         if (!(qm & blk) && (qm & ~(low | allowed)) == 0 && __builtin_popcountll(L | qm) <= pp.m) {
             L |= qm;
-            tr.ops.push_back((int)i);
+            tr.ops.push_back(i);
             take = true;
         } else if (!(qm & blk) && pp.hi_diag) {
             // a controlled phase with its control local (already, or added if it fits) and
@@ -196,7 +198,7 @@ Trial greedy_pass(const std::vector<OpInfo> &ops, const std::vector<char> &done,
             }
             if (q1) {
                 L |= q1 & (~q1 + 1ull);
-                tr.ops.push_back((int)i);
+                tr.ops.push_back(i);
                 take = true;
             }
         }
@@ -207,30 +209,44 @@ Trial greedy_pass(const std::vector<OpInfo> &ops, const std::vector<char> &done,
         if ((blocked & all) == all) break;
     }
     tr.L = L;
-    return tr;
 }
 
 }  // namespace
 
-std::vector<Pass> make_plan(const std::vector<Op> &ops, int n, const PlanParams &pp) {
+namespace {
+
+// The greedy partition, pass by pass, so that a comparison of two plans can stop early.
+struct PlanBuilder {
+    const std::vector<Op> &ops;
+    const int n;
+    const PlanParams &pp;
     std::vector<Pass> plan;
-    const uint64_t all = (n >= 64) ? ~0ull : ((1ull << n) - 1ull);
-    const int free_slots = pp.m - pp.c;
-    std::vector<char> done(ops.size(), 0);
-    const std::vector<OpInfo> info = op_info(ops, pp);
-    size_t first = 0;
-    while (first < ops.size()) {
-        while (first < ops.size() && done[first]) first++;
-        if (first >= ops.size()) break;
+    std::vector<char> done;
+    std::vector<OpInfo> open;  // ops in no pass yet
+    Trial best, t;
+
+    PlanBuilder(const std::vector<Op> &o, int n_qubits, const PlanParams &p)
+        : ops(o), n(n_qubits), pp(p), done(o.size(), 0), open(op_info(o, p)) {}
+
+    // Adds passes until every op is in one (true) or the plan has `limit` passes.
+    bool run(size_t limit) {
+        while (!open.empty() && plan.size() < limit) next();
+        return open.empty();
+    }
+
+    void next() {
+        const uint64_t all = (n >= 64) ? ~0ull : ((1ull << n) - 1ull);
+        const int free_slots = pp.m - pp.c;
+        const int first = open.front().index;
         // candidates: unrestricted greedy, and greedy restricted to each window of
         // free_slots consecutive high qubits (chains and brickwork advance further when the
         // local window is chosen, not claimed by the first gates in circuit order)
-        Trial best = greedy_pass(info, done, first, n, pp, all);
+        greedy_pass(open, n, pp, all, best);
         if (!best.stream && free_slots > 0 && n > pp.m) {
             for (int s = pp.c; s + free_slots <= n; s++) {
                 const uint64_t win = ((1ull << free_slots) - 1ull) << s;
-                Trial t = greedy_pass(info, done, first, n, pp, win);
-                if (!t.stream && t.ops.size() > best.ops.size()) best = std::move(t);
+                greedy_pass(open, n, pp, win, t);
+                if (!t.stream && t.ops.size() > best.ops.size()) std::swap(best, t);
             }
         }
         Pass pass;
@@ -239,9 +255,11 @@ std::vector<Pass> make_plan(const std::vector<Op> &ops, int n, const PlanParams 
         if (pass.ops.empty()) {
             // nothing fits next to the always-local low qubits (tiny m): stream the op
             pass.stream = true;
-            pass.ops.push_back((int)first);
+            pass.ops.push_back(first);
         }
-        for (int i : pass.ops) done[i] = 1;
+        for (int i : pass.ops) done[(size_t)i] = 1;
+        open.erase(std::remove_if(open.begin(), open.end(), [&](const OpInfo &op) { return done[(size_t)op.index] != 0; }),
+                   open.end());
         if (!pass.stream) {
             uint64_t L = best.L;
             // pad with the lowest free qubits (longer contiguous runs)
@@ -251,31 +269,41 @@ std::vector<Pass> make_plan(const std::vector<Op> &ops, int n, const PlanParams 
         }
         plan.push_back(std::move(pass));
     }
-    return plan;
+};
+
+}  // namespace
+
+std::vector<Pass> make_plan(const std::vector<Op> &ops, int n, const PlanParams &pp) {
+    PlanBuilder b(ops, n, pp);
+    b.run(SIZE_MAX);
+    return std::move(b.plan);
 }
 
 std::vector<Pass> choose_plan(const std::vector<Op> &ops, int n, const PlanParams &pp, const qs_options &o,
                               std::vector<Op> &merged, std::vector<std::pair<size_t, size_t>> &origin) {
     // Merged diagonal runs (one phase-function pass each) help where a run reaches more
     // qubits than a chunk pass holds (QAOA cost layers); chains of local diagonals are
-    // cheaper inside chunk passes (TFIM).  Both plans are built; the one with fewer passes
-    // over the state is run.
+    // cheaper inside chunk passes (TFIM).  The plan with fewer passes over the state is run,
+    // the merged one at equal counts (one table lookup per amplitude costs less FP64 work than
+    // the same gates as diagonal blocks inside chunk passes); neither is built further than
+    // it takes to know which.
     merged.clear();
     origin.clear();
-    std::vector<Pass> plan = make_plan(ops, n, pp);
-    if ((o.flags & QS_OPT_NO_DIAG_MERGE) != 0 || !phasefn_supported(n)) return plan;
+    PlanBuilder plain(ops, n, pp);
+    if ((o.flags & QS_OPT_NO_DIAG_MERGE) != 0 || !phasefn_supported(n)) {
+        plain.run(SIZE_MAX);
+        return std::move(plain.plan);
+    }
     std::vector<std::pair<size_t, size_t>> org;
     std::vector<Op> m = merge_diagonal_runs(ops, kMinMergedRun, &org);
-    if (m.size() >= ops.size()) return plan;
     // each phase function is a streaming pass of its own (not chunkable): the merged plan
     // has at least that many passes, plus one if any other op is left
     size_t n_pf = 0;
     for (const Op &op : m) n_pf += op.kind == K_PHASEFN;
-    if (n_pf + (m.size() > n_pf ? 1 : 0) > plan.size()) return plan;
+    const size_t least = m.size() >= ops.size() ? SIZE_MAX : n_pf + (m.size() > n_pf ? 1 : 0);
+    if (plain.run(least) && plain.plan.size() < least) return std::move(plain.plan);
     std::vector<Pass> alt = make_plan(m, n, pp);
-    // equal pass counts: the merged runs (one table lookup per amplitude) cost less FP64
-    // work than the same gates as diagonal blocks inside chunk passes
-    if (alt.size() > plan.size()) return plan;
+    if (plain.run(alt.size()) && plain.plan.size() < alt.size()) return std::move(plain.plan);
     merged = std::move(m);
     origin = std::move(org);
     return alt;
