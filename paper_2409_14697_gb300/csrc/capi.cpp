@@ -155,6 +155,7 @@ void run_circuit(DeviceState &d, const std::vector<Op> &ops, const qs_options &o
     d.prec = o.precision == QS_PREC_DF32 ? QS_PREC_DF32 : QS_PREC_FP64;
     d.ix = o.precision == QS_PREC_IX64 || o.precision == QS_PREC_DEFAULT;
     d.reg_phases = (o.flags & QS_OPT_NO_REG_PHASES) == 0;
+    d.drift = RoundingDrift{};
     const uint64_t l0 = g_launches.load();
     arena_begin(d);
     const int mode = o.mode;
@@ -394,6 +395,7 @@ int qs_plan(int n_qubits, qs_dtype dt, const qs_gate *gates, size_t n_gates, con
     d.n = n_qubits;
     d.dtype = dt;
     d.reg_phases = (o.flags & QS_OPT_NO_REG_PHASES) == 0;
+    d.drift = RoundingDrift{};
     std::vector<Op> merged;
     std::vector<std::pair<size_t, size_t>> origin;
     const std::vector<Pass> plan = choose_plan(ops, n_qubits, plan_params(d, o), o, merged, origin);

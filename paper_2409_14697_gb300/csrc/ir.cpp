@@ -308,6 +308,89 @@ std::vector<Op> split_one_qubit_phases(const std::vector<Op> &ops) {
     return out;
 }
 
+std::vector<Op> split_register_phases(std::vector<Op> ops) {
+    // u = diag(p0, p1) [[A, -S], [S, A]] diag(1, q1) with A = |a|, S = |c|; every unitary has
+    // this form, others are kept where it does not reproduce u
+    struct Parts {
+        cd p0, p1, q1;
+        double A, S;
+    };
+    auto split = [](const std::vector<cd> &u, Parts &r) {
+        const cd a = u[0], b = u[1], c = u[2], d = u[3];
+        r.A = std::abs(a);
+        r.S = std::abs(c);
+        if (r.A == 0.0 || r.S == 0.0) return false;
+        r.p0 = a / r.A;
+        r.p1 = c / r.S;
+        r.q1 = -b / (r.p0 * r.S);
+        const double tol = 1e-14;
+        return std::abs(std::abs(r.q1) - 1.0) <= tol && std::abs(r.p1 * r.q1 * r.A - d) <= tol;
+    };
+    int splittable = 0;
+    std::vector<char> can(ops.size(), 0);
+    std::vector<Parts> parts(ops.size());
+    // diagonal neighbour on the qubit before and after each one-qubit gate
+    std::vector<char> before(ops.size(), 0), after(ops.size(), 0);
+    int prev[64];
+    std::fill(prev, prev + 64, -1);
+    for (size_t i = 0; i < ops.size(); i++) {
+        const Op &op = ops[i];
+        const bool diag = op_is_diagonal(op);
+        for (int j = 0; j < op.k; j++) {
+            const int p = prev[op.q[j]];
+            if (p >= 0) {
+                before[i] |= op_is_diagonal(ops[(size_t)p]);
+                after[(size_t)p] |= diag;
+            }
+            prev[op.q[j]] = (int)i;
+        }
+        if (op.kind != K_DENSE1) continue;
+        const int32_t cls = d1_class(op.m);
+        if (cls == D1_REAL || !split(op.m, parts[i])) continue;
+        can[i] = cls == D1_RX ? 2 : 1;
+        splittable += can[i] == 1;
+    }
+    if (splittable < kMinSplitGates) splittable = 0;
+    std::vector<Op> out;
+    out.reserve(2 * ops.size());
+    int phase_at[64];  // one-qubit phase in `out` that later phases of the qubit may join
+    std::fill(phase_at, phase_at + 64, -1);
+    auto phase = [&](int q, cd d0, cd d1) {
+        if (phase_at[q] >= 0) {
+            Op &o = out[(size_t)phase_at[q]];
+            o.m = {o.m[0] * d0, o.m[1] * d1};
+            return;
+        }
+        Op o;
+        o.kind = K_DIAG1;
+        o.k = 1;
+        o.q[0] = q;
+        o.m = {d0, d1};
+        phase_at[q] = (int)out.size();
+        out.push_back(std::move(o));
+    };
+    for (size_t i = 0; i < ops.size(); i++) {
+        Op &op = ops[i];
+        const bool take = (can[i] == 1 && splittable) || (can[i] == 2 && before[i] && after[i]);
+        if (take) {
+            const int q = op.q[0];
+            const Parts &r = parts[i];
+            if (r.q1 != cd(1.0)) phase(q, 1.0, r.q1);
+            op.m = {cd(r.A), cd(-r.S), cd(r.S), cd(r.A)};
+            out.push_back(std::move(op));
+            phase_at[q] = -1;
+            phase(q, r.p0, r.p1);
+        } else if (op.kind == K_DIAG1 && splittable) {
+            phase(op.q[0], op.m[0], op.m[1]);
+        } else {
+            if (!op_is_diagonal(op))
+                for (int j = 0; j < op.k; j++) phase_at[op.q[j]] = -1;
+            out.push_back(std::move(op));
+        }
+    }
+    return out;
+}
+
 double op_flops(const Op &op) {
     // FP64 operations per amplitude of the one-qubit forms (general 8, real first entry 7,
     // real 4, RX-like 4)

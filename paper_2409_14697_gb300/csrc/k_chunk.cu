@@ -14,6 +14,7 @@
 #include <type_traits>
 
 #include "chunk.h"
+#include "kgeom.h"
 #include "kops.cuh"
 #include "ptx.cuh"
 #include "tile_ops.cuh"
@@ -22,8 +23,8 @@ namespace qs {
 namespace {
 
 constexpr int kChunkThreads = kTileThreads;
-// Dynamic shared memory of a staged pass (tile + program): two CTAs per SM must fit.
-constexpr size_t kStagedSmemLimit = 104 * 1024;
+// Shared memory an SM gives its resident CTAs, and what it keeps for each of them.
+constexpr size_t kSmemPerSm = 228 * 1024, kSmemPerCta = 1024;
 
 // Global amplitude index of tile t with its local bits zero.
 __device__ __forceinline__ uint64_t tile_base(uint64_t t, const ChunkArgs &a) {
@@ -111,8 +112,8 @@ __device__ void fold_hi_terms(const KOp &op, const T *src, T *dst, uint64_t base
 
 // DF: complex128 with double-float arithmetic; mats then holds (hi, lo) float pairs.
 // IX: complex128 one-qubit dense ops and constant diagonal ops in integer products
-// (QS_PREC_IX64).
-template <typename T, bool DF, bool IX>
+// (QS_PREC_IX64).  LAYERS: complex64 register phases in layers (pack_register_phases).
+template <typename T, bool DF, bool IX, bool LAYERS>
 __global__ void __launch_bounds__(kChunkThreads, 2)
 k_chunk(typename C2T<T>::type *__restrict__ psi, const ChunkArgs a, const KOp *__restrict__ ops,
         const T *__restrict__ mats, int *__restrict__ err) {
@@ -121,8 +122,9 @@ k_chunk(typename C2T<T>::type *__restrict__ psi, const ChunkArgs a, const KOp *_
     V *tile = (V *)smem_raw;
     __shared__ uint64_t bar;
     __shared__ int abort_flag;
+    __shared__ uint64_t s_run[kChunkThreads], s_base;
     __shared__ KOp s_op;
-    __shared__ T s_m[kMaxOpReals];
+    __shared__ __align__(16) T s_m[kMaxOpReals];
     __shared__ double s_fb[DF ? kMaxOpReals : 1];
     const uint32_t nruns = 1u << (a.m - a.c0);
     const uint32_t run_bytes = (uint32_t)sizeof(V) << a.c0;
@@ -144,16 +146,24 @@ k_chunk(typename C2T<T>::type *__restrict__ psi, const ChunkArgs a, const KOp *_
         T *dm = (T *)(smem_raw + a.reals_off);
         for (uint32_t j = threadIdx.x; j < a.n_reals; j += blockDim.x) dm[j] = mats[j];
     }
+    // where run r of a tile starts, the same for every tile (a pass with more runs computes it)
+    auto run_offset = [&](uint32_t r) {
+        uint64_t off = 0;
+        for (int j = 0; j < a.nlh; j++) off |= (uint64_t)((r >> j) & 1u) << a.lhigh[j];
+        return off;
+    };
+    if (nruns <= kChunkThreads && threadIdx.x < nruns) s_run[threadIdx.x] = run_offset(threadIdx.x);
     __syncthreads();
     uint32_t phase = 0;
     for (uint64_t t = blockIdx.x; t < a.n_tiles; t += gridDim.x) {
-        uint64_t base = tile_base(t, a);
-        if (threadIdx.x == 0) ptx::mbar_arrive_expect_tx(&bar, tile_bytes);
+        if (threadIdx.x == 0) {
+            s_base = tile_base(t, a);
+            ptx::mbar_arrive_expect_tx(&bar, tile_bytes);
+        }
         __syncthreads();
         for (uint32_t r = threadIdx.x; r < nruns; r += blockDim.x) {
-            uint64_t off = 0;
-            for (int j = 0; j < a.nlh; j++) off |= (uint64_t)((r >> j) & 1u) << a.lhigh[j];
-            ptx::bulk_g2s(tile + ((uint64_t)r << a.c0), psi + (base | off), run_bytes, &bar);
+            const uint64_t off = nruns <= kChunkThreads ? s_run[r] : run_offset(r);
+            ptx::bulk_g2s(tile + ((uint64_t)r << a.c0), psi + (s_base | off), run_bytes, &bar);
         }
         if (!ptx::mbar_wait_bounded(&bar, phase, ptx::kWaitLimitNs)) {
             abort_flag = 1;
@@ -187,12 +197,12 @@ k_chunk(typename C2T<T>::type *__restrict__ psi, const ChunkArgs a, const KOp *_
             }
             if constexpr (std::is_same<T, double>::value) {  // complex128 passes only
                 if ((op->fkind == F_CDIAGK || op->fkind == F_HCDIAGK) && op->nt > 0) {
-                    fold_hi_terms<DF>(*op, om, s_m, tile_base(t, a));
+                    fold_hi_terms<DF>(*op, om, s_m, s_base);
                     om = s_m;
                 }
             }
             if constexpr (DF) apply_op_dftile((double2 *)tile, *op, (const df::F2 *)om, s_fb, a.m);
-            else apply_op_smem<T, true, IX>(tile, *op, om, a.m);
+            else apply_op_smem<T, true, IX, LAYERS>(tile, *op, om, a.m);
             __syncthreads();
         }
         if constexpr (DF) {
@@ -201,14 +211,9 @@ k_chunk(typename C2T<T>::type *__restrict__ psi, const ChunkArgs a, const KOp *_
         }
         ptx::fence_proxy_async_smem();
         __syncthreads();
-        // the write-back addresses are rebuilt rather than kept live through the ops
-        // (register pressure of the complex64 register phases)
-        asm volatile("" ::: "memory");
-        base = tile_base(t, a);
         for (uint32_t r = threadIdx.x; r < nruns; r += blockDim.x) {
-            uint64_t off = 0;
-            for (int j = 0; j < a.nlh; j++) off |= (uint64_t)((r >> j) & 1u) << a.lhigh[j];
-            ptx::bulk_s2g(psi + (base | off), tile + ((uint64_t)r << a.c0), run_bytes);
+            const uint64_t off = nruns <= kChunkThreads ? s_run[r] : run_offset(r);
+            ptx::bulk_s2g(psi + (s_base | off), tile + ((uint64_t)r << a.c0), run_bytes);
         }
         ptx::bulk_commit();
         ptx::bulk_wait_read_all();
@@ -217,7 +222,18 @@ k_chunk(typename C2T<T>::type *__restrict__ psi, const ChunkArgs a, const KOp *_
     ptx::bulk_wait_all();
 }
 
-template <typename T, bool DF, bool IX>
+// Dynamic shared memory of a staged pass (tile + program): two CTAs per SM must fit beside the
+// kernel's own arrays.
+template <typename T, bool DF, bool IX, bool LAYERS = false> size_t staged_limit() {
+    static const size_t limit = [] {
+        cudaFuncAttributes at{};
+        QS_CUDA(cudaFuncGetAttributes(&at, k_chunk<T, DF, IX, LAYERS>));
+        return (kSmemPerSm / 2 - kSmemPerCta - at.sharedSizeBytes) / 128 * 128;
+    }();
+    return limit;
+}
+
+template <typename T, bool DF, bool IX, bool LAYERS = false>
 void launch_t(DeviceState &st, const ChunkArgs &a, const std::vector<KOp> &kops, const std::vector<double> &mats) {
     const KOp *d_ops = (const KOp *)upload_params(st, kops.data(), kops.size() * sizeof(KOp));
     const T *d_m;
@@ -244,9 +260,9 @@ void launch_t(DeviceState &st, const ChunkArgs &a, const std::vector<KOp> &kops,
     ca.ops_off = (uint32_t)tile_bytes;
     ca.reals_off = (uint32_t)(tile_bytes + ops_bytes);
     ca.n_reals = (uint32_t)mats.size();
-    ca.staged = tile_bytes + ops_bytes + reals_bytes <= kStagedSmemLimit ? 1 : 0;
+    ca.staged = tile_bytes + ops_bytes + reals_bytes <= staged_limit<T, DF, IX, LAYERS>() ? 1 : 0;
     if (ca.staged) smem = (tile_bytes + ops_bytes + reals_bytes + 15) / 16 * 16;
-    auto kern = k_chunk<T, DF, IX>;
+    auto kern = k_chunk<T, DF, IX, LAYERS>;
     static bool attr_set = false;
     if (!attr_set) {
         QS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
@@ -283,7 +299,17 @@ void launch_chunk_pass(DeviceState &st, uint64_t lmask, const std::vector<KOp> &
         else if (st.ix) launch_t<double, false, true>(st, a, kops, mats);
         else launch_t<double, false, false>(st, a, kops, mats);
     } else {
-        launch_t<float, false, false>(st, a, kops, mats);
+        bool phases = false;
+        for (const KOp &k : kops) phases |= k.fkind == F_RPHASE;
+        const size_t taken = (B << a.m) + kops.size() * sizeof(KOp);
+        const size_t limit = staged_limit<float, false, false, true>();
+        if (phases && n - a.m >= kPackTileBits && taken < limit) {
+            std::vector<double> packed;
+            const std::vector<KOp> pk = pack_register_phases(kops, mats, (limit - taken) / sizeof(float), packed, &st.drift);
+            launch_t<float, false, false, true>(st, a, pk, packed);
+        } else {
+            launch_t<float, false, false>(st, a, kops, mats);
+        }
     }
 }
 

@@ -397,7 +397,7 @@ uint32_t tile_mask(const Op &op, const int *pos) {
 bool rphase_applicable(int m, int thread_bits) { return m - thread_bits == kRpBits; }
 
 std::vector<KOp> build_register_phases(const std::vector<Op> &ops, const int *pos, int m, int thread_bits,
-                                       std::vector<double> &mats, int *n_phases) {
+                                       std::vector<double> &mats, int *n_phases, bool layered) {
     if (!rphase_applicable(m, thread_bits)) fail(QS_ERR_INVALID, "register phases need m = thread bits + 5");
     const size_t N = ops.size();
     std::vector<RpMember> mb(N);
@@ -456,6 +456,25 @@ std::vector<KOp> build_register_phases(const std::vector<Op> &ops, const int *po
                 best.swap(cand);
                 R = Rw;
             }
+        }
+        // a diagonal that no matrix of this phase follows waits for the phase that brings one of
+        // its positions into registers (there it joins a table), if a gate that is not diagonal
+        // is left on them; plain phases keep those on a register position
+        uint32_t later = 0, next = 0;
+        {
+            std::vector<char> taken(N, 0);
+            for (int i : best) taken[i] = 1;
+            for (int i : open)
+                if (!taken[i] && !diag[i]) later |= touch[i];
+            cand.clear();
+            for (size_t k = best.size(); k-- > 0;) {  // next: positions that a later matrix changes
+                const int i = best[k];
+                const bool used = layered ? (touch[i] & next) != 0 : (touch[i] & R) != 0;
+                if (!diag[i]) next |= 1u << mb[i].tgt;
+                if (!diag[i] || used || !(touch[i] & later)) cand.push_back(i);
+            }
+            std::reverse(cand.begin(), cand.end());
+            if (!cand.empty()) best.swap(cand);
         }
         // pad R with the highest free positions
         for (int p = m - 1; p >= 0 && __builtin_popcount(R) < kRpBits; p--) R |= 1u << p;

@@ -30,7 +30,20 @@ bool rphase_applicable(int m, int thread_bits);
 // (swaps, wider dense or diagonal blocks) become ordinary KOps in their place in the
 // order.  n_phases (optional) receives the number of phases.
 std::vector<KOp> build_register_phases(const std::vector<Op> &ops, const int *pos, int m, int thread_bits,
-                                       std::vector<double> &mats, int *n_phases = nullptr);
+                                       std::vector<double> &mats, int *n_phases = nullptr, bool layered = false);
+
+// Passes of 2^kPackTileBits tiles or more run their register phases in layers, with one-qubit
+// gates split into rotations and phases; smaller states wait for the host, which takes about
+// 60 us longer per pass to build them (20-layer brickwork, 21 qubits: 0.76 ms against 0.60; 22
+// qubits: 0.81 against 0.96).
+constexpr int kPackTileBits = 9;
+// A pass's register phases in layers: layers of a factor table and real matrices (rphase.cpp).
+// Returns the ops with their reals re-laid in `out` (other ops unchanged), which stays within
+// max_reals, if it can, by giving later phases one layer of their members as they are; every
+// phase starts at a multiple of 4 reals.  drift: the call's account of what rounding to FP32 did
+// to the norm; none: tables are not corrected for it.
+std::vector<KOp> pack_register_phases(const std::vector<KOp> &kops, const std::vector<double> &mats, size_t max_reals,
+                                      std::vector<double> &out, RoundingDrift *drift = nullptr);
 
 // Fraction of the state's bytes one streaming application reads and writes, counting
 // whole DRAM sectors of 2^sector_bits elements.

@@ -55,7 +55,7 @@ constexpr int kTileThreads = 1 << kTileThreadBits;
 constexpr int kRpBits = 5;
 constexpr int kRpAlways = 31;     // position operand whose bit is 1 for every amplitude
 constexpr int kRpNever = 30;      // position operand whose bit is 0 for every amplitude
-constexpr int kRpMaxMembers = 56; // ops per phase: 1 + 9 * 56 reals <= kMaxOpReals
+constexpr int kRpMaxMembers = 56; // ops per phase: 8 + 9 * 56 reals <= kMaxOpReals
 enum RpType : int {
     RP_M1 = 0,  // 2x2 matrix on register slot `slot`; operand b holds its form: RP_GENERAL
                 // (8 reals, row-major re, im), RP_REAL (4 reals: m00 m01 m10 m11; H, RY) or
@@ -73,6 +73,18 @@ enum RpType : int {
     RP_PARITYN, // np parity patterns (a | b << 5), then np + 1 factors (re, im) indexed by the
                 // number of patterns with x_a != x_b (equal-angle RZZ / RZ layers), np <= 15
 };
+// Phases in layers (pack_register_phases): the number of layers and three unused reals,
+// then the layers, then the tables.  A layer is
+//   h0 = real slots | class bits b << 10 | table << 13,
+//   h1 = offset of its table from the program's start, h2 = the b thread-index bits that spell
+//   a thread's class c (4 bits each, bit i of c <-> i-th), h3 = members | their reals / 4 << 8,
+// then 8 reals per real slot (a real 2x2 matrix, row-major, and X M X for lanes whose bit of
+// sigma is set), then the other members (as above) up to a multiple of 4 reals; applied in this
+// order.  Table: register r takes the complex factor at ((r >> 1) 2^b + c) 4 + 2 (r & 1).  An
+// RP_DIAG member with slot field 1 and payload
+// (offset, lo, hi) multiplies every register by the factor at 2 c of a table, c of `a` bits named
+// 4 bits each in lo and hi.
+constexpr int kRpMaxClassBits = 4;  // at most 16 classes (a table of 4 KiB)
 constexpr int kRpMaxParity = 15;
 // Run form of RP_PH: at most 31 phases and 31 sign pairs (5-bit counts); below
 // kRpMinRunPhases phases the separate members cost less.

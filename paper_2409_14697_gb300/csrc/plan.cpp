@@ -58,7 +58,8 @@ int launch_pass_ops(DeviceState &st, uint64_t lmask, const std::vector<Op> &fuse
     std::vector<KOp> kops;
     std::vector<double> mats;
     if (!use_tc && st.dtype == QS_C64 && st.reg_phases && rphase_applicable(m, kTileThreadBits)) {
-        const std::vector<KOp> kp = build_register_phases(fused, pos, m, kTileThreadBits, mats);
+        const std::vector<KOp> kp = build_register_phases(fused, pos, m, kTileThreadBits, mats, nullptr,
+                                                           n - m >= kPackTileBits);
         launch_chunk_pass(st, lmask, kp, mats);
         return (int)kp.size();
     }
@@ -317,10 +318,9 @@ std::vector<Op> pass_program(const DeviceState &st, const PlanParams &pp, const 
     if (st.dtype == QS_C128) defer_hadamard_scale(pops);
     std::vector<Op> fused = fuse_ops(std::move(pops), pp.fuse_k, pp.sweep_flops, p.lmask);
     if (st.dtype == QS_C128 && st.prec == QS_PREC_FP64 && st.n - local >= 8) fused = split_one_qubit_phases(fused);
-    // (complex64 register phases keep U3 whole: split into a rotation between phases, with
-    // the phases joined in run members, the 33-qubit brickwork took 5.77 s against 4.77 s)
     const bool phases = st.dtype == QS_C64 && st.reg_phases && !pp.tc && rphase_applicable(local, kTileThreadBits);
-    if (!phases)
+    if (phases && st.n - local >= kPackTileBits) fused = split_register_phases(std::move(fused));
+    else if (!phases)
         fused = merge_tile_diagonals(std::move(fused), kTileDiagQubits, st.dtype == QS_C128 ? 0.5 : 4.0,
                                      pp.hi_diag ? p.lmask : 0);
     return fused;

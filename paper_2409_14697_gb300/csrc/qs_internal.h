@@ -131,6 +131,13 @@ void defer_hadamard_scale(std::vector<Op> &ops);
 // gates (a CZ layer) in one run that merge_tile_diagonals applies as a few table
 // multiplies.  Ops whose matrix the split does not reproduce to 1e-14 are kept.
 std::vector<Op> split_one_qubit_phases(const std::vector<Op> &ops);
+// The same for complex64 register phases, where a real 2x2 is the cheapest matrix and every
+// run of diagonals costs one table multiply (rphase.cpp): one-qubit unitaries as a real
+// rotation between phases diag(p0, p1) and diag(1, q1), adjacent phases of a qubit joined.  A
+// pass of fewer than kMinSplitGates such gates keeps them whole (it is bound by HBM); RX-like
+// matrices, which already cost as little as a real one, are split only between diagonals.
+std::vector<Op> split_register_phases(std::vector<Op> ops);
+constexpr int kMinSplitGates = 8;
 // Structure class (D1_GENERAL, D1_R0, D1_REAL, D1_RX of kops.cuh) of a 2x2 matrix,
 // row-major: the cheapest form the complex128 kernels apply it with.
 int32_t d1_class(const std::vector<cd> &u);
@@ -158,6 +165,14 @@ constexpr int kArenas = 16;
 
 // Tensor Product Booster: most groups of one product pass (k_tpb.cu, tpb.cpp).
 constexpr int kTpbMaxGroups = 4;
+
+// What rounding matrices and tables to FP32 did to the norm of a state in one call (complex64
+// register phases): logarithms of what is open, and of what tables have been scaled by for it
+// (at most kMaxDriftFix in all).
+constexpr double kMaxDriftFix = 6e-6;
+struct RoundingDrift {
+    double open = 0.0, fixed = 0.0;
+};
 
 struct DeviceState {
     void *psi = nullptr;  // amplitudes
@@ -188,6 +203,7 @@ struct DeviceState {
     // the amplitudes are |0...0> (set by launch_set_zero_state; cleared by every other
     // write): qs_apply_circuit may then build a prefix as a tensor product
     bool known_zero = false;
+    RoundingDrift drift;  // of the running call
     // Tensor Product Booster: group sub-states (small states of their own) and their memory
     DeviceState *tpb_sub[kTpbMaxGroups] = {};
     void *tpb_buf = nullptr;

@@ -1,0 +1,589 @@
+// Host: packing of complex64 register-phase programs for the device.
+//
+// build_register_phases (kgeom.cpp) gives each phase a list of members in circuit order:
+// one-qubit matrices, controlled matrices and exchanges on register slots, and diagonals on
+// any positions.  Applied one by one the diagonals cost the phase more than its matrices
+// (every equal-angle RZZ run counts bit patterns per register, every run of one-qubit
+// phases builds factor tables per thread).  But which factor register r of thread t takes
+// from a run of diagonals depends on the thread only through a few bits of its index: the
+// partners of two-qubit diagonals outside the register slots, and the lane bits that permute
+// the register order (sigma).  So the run becomes one table of 2^5 factors for every value
+// ("class") of those bits, made here in FP64, and one complex multiply per amplitude on
+// the device whatever the number of gates.
+//
+// Members commute unless one changes a position that the other uses, so the list is first
+// rescheduled: matrices as early as their slots' diagonals allow, diagonals gathered in as few
+// runs as the matrices between them allow.  The result is a list of layers, each a table, then
+// real 2x2 matrices on different slots, then other members as they were: the device reads one
+// header per layer, where a member by itself cost about as many instructions to read as a
+// real matrix costs to apply.
+//
+// The device's reals are FP32, and the rounding of an angle that a circuit repeats (Trotter
+// steps) changes the norm the same way each time.  What the matrices and the tables so far have
+// changed it by is divided out of the next table, whose own rounding then joins the account
+// (RoundingDrift): the 25-qubit Trotter circuit of 16 steps ended up to 1.1e-5 off, now 5e-7.
+// A call never divides out more than kMaxDriftFix, so that its result also stays as near to what
+// the plain FP32 matrices of the other execution modes give.
+#include <algorithm>
+#include <cmath>
+
+#include "kgeom.h"
+
+namespace qs {
+namespace {
+
+constexpr int kThreadBits = kTileThreadBits;  // position ids 0..7: thread-index bits, 8..12: slots
+constexpr int kRegs = 1 << kRpBits;
+constexpr uint32_t kSlotMask = ((1u << kRpBits) - 1u) << kThreadBits;
+
+// One diagonal factor on at most two positions (ids ascending): d[x0 + 2 x1].
+struct Term {
+    int np = 0;
+    int pos[2] = {-1, -1};
+    cd d[4] = {1.0, 1.0, 1.0, 1.0};
+    bool sign = false;  // only factors 1 and -1, from a sign member
+    int lo = 0, hi = 0, at = -1;
+    uint32_t mask() const { return (np > 0 ? 1u << pos[0] : 0u) | (np > 1 ? 1u << pos[1] : 0u); }
+};
+
+// A matrix, controlled matrix or exchange, kept as it is encoded.
+struct Matrix {
+    const double *code;
+    int len;
+    int slot, ctl;  // ctl: operand encoding of the control, -1 if none
+    bool exchange, real;
+    int at = 0;
+};
+
+// sigma bit of a slot as an affine function of the thread index
+struct Sigma {
+    uint32_t bits = 0;
+    bool one = false;
+};
+
+constexpr int kNone = -1, kOn = -2, kOff = -3;
+// operand encoding -> position id, kOn (bit 1 everywhere) or kOff
+int position_of(int enc) {
+    if (enc == kRpAlways) return kOn;
+    if (enc == kRpNever) return kOff;
+    return (enc & 16) ? kThreadBits + (enc & 15) : enc;
+}
+
+// Encoding of a position id in a member.
+int encode_position(int id) {
+    if (id < 0) return kRpAlways;
+    return id >= kThreadBits ? 16 + (id - kThreadBits) : id;
+}
+
+// A term from a function f(x_a, x_b) of two operand encodings.
+template <typename F> Term make_term(int ea, int eb, const F &f) {
+    Term t;
+    const int a = position_of(ea), b = position_of(eb);
+    auto value = [](int p, int id, int x) { return p == kOn ? 1 : p == kOff ? 0 : p == id ? x : 0; };
+    if (a >= 0) t.pos[t.np++] = a;
+    if (b >= 0 && b != a) t.pos[t.np++] = b;
+    if (t.np == 2 && t.pos[0] > t.pos[1]) std::swap(t.pos[0], t.pos[1]);
+    for (int x = 0; x < 4; x++) {
+        const int x0 = x & 1, x1 = x >> 1;
+        const int va = a >= 0 ? (a == t.pos[0] ? x0 : x1) : value(a, a, 0);
+        const int vb = b >= 0 ? (b == t.pos[0] ? x0 : x1) : value(b, b, 0);
+        t.d[x] = f(va, vb);
+    }
+    return t;
+}
+
+// Logarithm of the factor by which rounding the reals of a 2x2 member to FP32 changes the norm.
+double rounding_drift(const Matrix &m) {
+    if (((int)m.code[0] & 7) != RP_M1) return 0.0;
+    double exact = 0.0, rounded = 0.0;
+    for (int i = 1; i < m.len; i++) {
+        const double v = m.code[i], f = (double)(float)v;
+        exact += v * v;
+        rounded += f * f;
+    }
+    return exact > 0.0 && rounded > 0.0 ? 0.5 * std::log1p((rounded - exact) / exact) : 0.0;
+}
+
+struct Packer {
+    const KOp &ph;
+    std::vector<Term> terms;
+    std::vector<Matrix> mats;
+    std::vector<std::pair<bool, int>> order;  // (is matrix, index) in circuit order
+    Sigma sigma[kRpBits];
+
+    explicit Packer(const KOp &p) : ph(p) {
+        int nlow = 0;
+        for (int j = 0; j < kRpBits; j++) nlow += ph.pos[j] < 4 ? 1 : 0;
+        int li = 4 - nlow;  // lane bits of the positions below 4, as rp_geometry assigns them
+        for (int j = 0; j < kRpBits; j++)
+            if (ph.pos[j] < 4) sigma[j].bits = 1u << li++;
+    }
+
+    void add(Term t) {
+        order.push_back({false, (int)terms.size()});
+        terms.push_back(t);
+    }
+
+    // false: a member this packing does not know
+    bool decode(const double *prog) {
+        const int nmem = (int)prog[0];
+        const double *mm = prog + 1;
+        for (int i = 0; i < nmem; i++) {
+            const int code = (int)mm[0];
+            const int type = code & 7, J = (code >> 3) & 7, ea = (code >> 6) & 31, eb = (code >> 11) & 31;
+            const int len = (code >> 16) & 255;
+            const double *P = mm + 1;
+            auto c = [&](int j) { return cd(P[2 * j], P[2 * j + 1]); };
+            switch (type) {
+            case RP_M1: case RP_C1: case RP_X:
+                order.push_back({true, (int)mats.size()});
+                mats.push_back({mm, 1 + len, J, type == RP_M1 ? -1 : ea, type == RP_X, type == RP_M1 && eb == RP_REAL});
+                break;
+            case RP_DIAG:
+                if (ea == eb) add(make_term(ea, ea, [&](int a, int) { return c(3 * a); }));
+                else add(make_term(ea, eb, [&](int a, int b) { return c(2 * a + b); }));
+                break;
+            case RP_NEG:
+                for (int q = 0; q <= J; q++) {
+                    const int e = (int)P[q];
+                    add(make_term(e & 31, e >> 5, [&](int a, int b) { return cd(a && b ? -1.0 : 1.0); }));
+                    terms.back().sign = true;
+                }
+                break;
+            case RP_PARITY:
+                add(make_term(ea, eb, [&](int a, int b) { return c(a ^ b); }));
+                break;
+            case RP_PARITYN: {
+                const int np = (len - 2) / 3;
+                const cd t0(P[np], P[np + 1]), t1(P[np + 2], P[np + 3]);
+                if (t0 == cd(0.0)) return false;
+                Term k;  // the factor of no odd pattern, then the step from one count to the next
+                for (cd &z : k.d) z = t0;
+                add(k);
+                const cd step = t1 / t0;
+                for (int q = 0; q < np; q++) {
+                    const int e = (int)P[q];
+                    add(make_term(e & 31, e >> 5, [&](int a, int b) { return a ^ b ? step : cd(1.0); }));
+                }
+                break;
+            }
+            default:  // RP_PH
+                if (J == 1) {
+                    for (int q = 0; q < ea; q++) {
+                        const int e = (int)P[3 * q];
+                        const cd z(P[3 * q + 1], P[3 * q + 2]);
+                        add(make_term(e, e, [&](int a, int) { return a ? z : cd(1.0); }));
+                    }
+                    for (int q = 0; q < eb; q++) {
+                        const int e = (int)P[3 * ea + q];
+                        add(make_term(e & 31, e >> 5, [&](int a, int b) { return cd(a && b ? -1.0 : 1.0); }));
+                        terms.back().sign = true;
+                    }
+                } else {
+                    add(make_term(ea, eb, [&](int a, int b) { return a && b ? c(0) : cd(1.0); }));
+                }
+                break;
+            }
+            mm += 1 + len;
+        }
+        return true;
+    }
+
+    // Times: diagonal runs at even times, matrices at odd ones.  Matrices as early as their
+    // operands allow; a term may go to any even time of [lo, hi].
+    void schedule() {
+        int changed[kThreadBits + kRpBits], read[kThreadBits + kRpBits];  // last time a position was ...
+        std::fill(changed, changed + kThreadBits + kRpBits, -1);
+        std::fill(read, read + kThreadBits + kRpBits, 0);
+        std::vector<int> open[kRpBits];  // terms on a slot since its last matrix
+        int last = 0;
+        for (const auto &o : order) {
+            if (!o.first) {
+                Term &t = terms[o.second];
+                t.lo = 0;
+                for (int k = 0; k < t.np; k++) t.lo = std::max(t.lo, changed[t.pos[k]] + 1);
+                t.hi = 1 << 20;
+                for (int k = 0; k < t.np; k++) {
+                    read[t.pos[k]] = std::max(read[t.pos[k]], t.lo);
+                    if (t.pos[k] >= kThreadBits) open[t.pos[k] - kThreadBits].push_back(o.second);
+                }
+                continue;
+            }
+            Matrix &m = mats[o.second];
+            const int s = kThreadBits + m.slot;
+            int t = std::max(changed[s], read[s] + 1);
+            const int c = m.ctl >= 0 ? position_of(m.ctl) : kNone;
+            if (c >= 0) t = std::max(t, changed[c]);
+            if (t % 2 == 0) t++;
+            m.at = t;
+            changed[s] = t;
+            // a control is read at an odd time: a later matrix on it may share that time (order
+            // is kept inside a time), a diagonal on it does not change it
+            if (c >= kThreadBits) read[c] = std::max(read[c], t - 1);
+            for (int i : open[m.slot]) terms[i].hi = std::min(terms[i].hi, t - 1);
+            open[m.slot].clear();
+            last = std::max(last, t);
+        }
+        // fewest runs: terms by their last time, each in the latest run already placed inside its
+        // interval, else in a new run at its last time
+        std::vector<int> by(terms.size());
+        for (size_t i = 0; i < by.size(); i++) by[i] = (int)i;
+        const int end = last ? last + 1 : 0;
+        for (Term &t : terms) t.hi = std::min(t.hi, end);
+        std::stable_sort(by.begin(), by.end(), [&](int a, int b) { return terms[a].hi < terms[b].hi; });
+        std::vector<int> runs;
+        for (int i : by) {
+            Term &t = terms[i];
+            if ((t.mask() & kSlotMask) == 0) continue;
+            for (int r : runs)
+                if (r >= t.lo && r <= t.hi) t.at = std::max(t.at, r);
+            if (t.at < 0) runs.push_back(t.at = t.hi);
+        }
+        // factors that no register position chooses: with any run
+        for (Term &t : terms)
+            if (t.at < 0) t.at = runs.empty() ? end : runs.back();
+    }
+};
+
+// A table under construction: the terms it takes and the thread bits that choose its class.
+struct Table {
+    std::vector<int> terms;
+    uint32_t bits = 0;
+};
+
+// Appends the 2^5 factors per class: factor of register r and class c at
+// ((r >> 1) 2^b + c) 4 + 2 (r & 1), so that a thread's loads are 16 bytes and threads of a
+// quarter-warp, which differ in the lowest thread bits, read neighbouring classes.
+// All of them are multiplied by `scale`; returns the sum of their squares as they are and as
+// FP32.
+std::pair<double, double> emit_table(const Packer &p, const Table &tb, double scale, std::vector<double> &out) {
+    int bit[kRpMaxClassBits], nb = 0;
+    for (int i = 0; i < kThreadBits; i++)
+        if ((tb.bits >> i) & 1u) bit[nb++] = i;
+    const size_t at = out.size();
+    out.resize(at + ((size_t)64 << nb));
+    // factors in logical order (slot bits x), real and imaginary parts
+    struct Factors {
+        double re[kRegs], im[kRegs];
+        void mul(int x, cd z) {
+            const double r = re[x] * z.real() - im[x] * z.imag();
+            im[x] = re[x] * z.imag() + im[x] * z.real();
+            re[x] = r;
+        }
+    };
+    Factors fixed;  // the part that only slots choose
+    std::fill(fixed.re, fixed.re + kRegs, scale);
+    std::fill(fixed.im, fixed.im + kRegs, 0.0);
+    std::vector<const Term *> mixed;
+    uint32_t chooses = 0;  // thread bits in terms (the others of the class only permute)
+    for (int i : tb.terms) {
+        const Term &t = p.terms[i];
+        if (t.np > 0 && t.pos[0] < kThreadBits) {
+            mixed.push_back(&t);
+            chooses |= t.mask();
+            continue;
+        }
+        const int a = t.np > 0 ? t.pos[0] - kThreadBits : 0, b = t.np == 2 ? t.pos[1] - kThreadBits : 0;
+        for (int x = 0; x < kRegs; x++)
+            fixed.mul(x, t.d[(t.np > 0 ? (x >> a) & 1 : 0) + (t.np == 2 ? 2 * ((x >> b) & 1) : 0)]);
+    }
+    Factors f = fixed;
+    double exact = 0.0, rounded = 0.0, exact_f = 0.0, rounded_f = 0.0;
+    auto weigh = [&]() {  // a class's factors, whatever their order
+        exact_f = rounded_f = 0.0;
+        for (int x = 0; x < kRegs; x++) {
+            const double r = (double)(float)f.re[x], i = (double)(float)f.im[x];
+            exact_f += f.re[x] * f.re[x] + f.im[x] * f.im[x];
+            rounded_f += r * r + i * i;
+        }
+    };
+    weigh();
+    uint32_t made = ~0u;  // the chosen bits that f was made for
+    for (int c = 0; c < (1 << nb); c++) {
+        uint32_t tid = 0;
+        for (int i = 0; i < nb; i++) tid |= (uint32_t)((c >> i) & 1) << bit[i];
+        if (!mixed.empty() && (tid & chooses) != made) {
+            made = tid & chooses;
+            f = fixed;
+            for (const Term *t : mixed) {
+                const int x0 = (tid >> t->pos[0]) & 1;
+                if (t->np == 2 && t->pos[1] >= kThreadBits) {
+                    const int j = t->pos[1] - kThreadBits;
+                    for (int h = 0; h < 2; h++)
+                        if (t->d[x0 + 2 * h] != cd(1.0))
+                            for (int x = 0; x < kRegs; x++)
+                                if (((x >> j) & 1) == h) f.mul(x, t->d[x0 + 2 * h]);
+                } else {
+                    const cd z = t->d[x0 + (t->np == 2 ? 2 * ((tid >> t->pos[1]) & 1) : 0)];
+                    for (int x = 0; x < kRegs; x++) f.mul(x, z);
+                }
+            }
+            weigh();
+        }
+        exact += exact_f;
+        rounded += rounded_f;
+        int sg = 0;  // register r holds the amplitude whose slot bits are r ^ sigma
+        for (int j = 0; j < kRpBits; j++)
+            sg |= (int)((__builtin_popcount(p.sigma[j].bits & tid) & 1) ^ (p.sigma[j].one ? 1 : 0)) << j;
+        double *o = out.data() + at + 4 * (size_t)c;
+        for (int r = 0; r < kRegs; r += 2, o += (size_t)4 << nb) {
+            o[0] = f.re[r ^ sg];
+            o[1] = f.im[r ^ sg];
+            o[2] = f.re[(r + 1) ^ sg];
+            o[3] = f.im[(r + 1) ^ sg];
+        }
+    }
+    return {exact, rounded};
+}
+
+// Appends the factor of every class for terms that no slot chooses, 2 reals each.
+void emit_thread_table(const Packer &p, const Table &tb, std::vector<double> &out) {
+    int at[kThreadBits] = {0}, nb = 0;
+    for (int i = 0; i < kThreadBits; i++)
+        if ((tb.bits >> i) & 1u) at[i] = nb++;
+    for (int c = 0; c < (1 << nb); c++) {
+        cd f = 1.0;
+        for (int i : tb.terms) {
+            const Term &t = p.terms[i];
+            const int x0 = t.np > 0 ? (c >> at[t.pos[0]]) & 1 : 0, x1 = t.np > 1 ? (c >> at[t.pos[1]]) & 1 : 0;
+            f *= t.d[x0 + 2 * x1];
+        }
+        out.push_back(f.real());
+        out.push_back(f.imag());
+    }
+    while (out.size() % 4) out.push_back(0.0);
+}
+
+// One layer of the packed program, in the device's order of execution.
+struct Layer {
+    int table = -1;      // index into the tables' offsets, -1: none
+    int class_bits = 0;  // number of thread bits that spell a class
+    uint32_t class_pos = 0;
+    const Matrix *real[kRpBits] = {nullptr};
+    int members = 0;          // other members, in order
+    std::vector<double> raw;
+    uint32_t raw_uses = 0;    // slots they change or read
+};
+
+// Packs one phase; the program goes to `out` at a multiple of 4 reals.  max_reals: what it may
+// take.  False: `out` is as before (no table to gain, an unknown member, or too long).
+bool pack_phase(const KOp &ph, const std::vector<double> &in, size_t max_reals, RoundingDrift *drift,
+                std::vector<double> &out, KOp &res) {
+    Packer p(ph);
+    if (ph.nt != kThreadBits || !p.decode(in.data() + ph.mat)) return false;
+    if (p.terms.empty()) return false;
+    p.schedule();
+    int last = 0;
+    for (const Matrix &m : p.mats) last = std::max(last, m.at);
+    for (const Term &t : p.terms) last = std::max(last, t.at);
+    RoundingDrift account = drift ? *drift : RoundingDrift{};
+    for (const Matrix &m : p.mats) account.open += rounding_drift(m);
+    std::vector<Layer> layers;
+    std::vector<double> tables;
+    std::vector<size_t> table_at;
+    auto raw = [&](int type, int slot, int ea, int eb, const std::vector<double> &pay) {
+        if (layers.empty()) layers.emplace_back();
+        Layer &l = layers.back();
+        l.members++;
+        l.raw.push_back((double)(type | slot << 3 | ea << 6 | eb << 11 | (int)pay.size() << 16));
+        l.raw.insert(l.raw.end(), pay.begin(), pay.end());
+        l.raw_uses = kSlotMask;  // a diagonal: nothing later may go before it
+    };
+    // terms by themselves: sign pairs are collected, other factors as a diagonal of their own
+    auto raw_terms = [&](const std::vector<int> &list) {
+        std::vector<double> pairs;
+        auto flush = [&]() {
+            if (!pairs.empty()) raw(RP_NEG, (int)pairs.size() - 1, 0, 0, pairs);
+            pairs.clear();
+        };
+        for (int i : list) {
+            const Term &t = p.terms[i];
+            const int a = t.np > 0 ? encode_position(t.pos[0]) : kRpAlways;
+            const int b = t.np > 1 ? encode_position(t.pos[1]) : a;
+            if (t.sign) {
+                // a sign member's term is -1 exactly where its one or two positions are 1, or
+                // nowhere (paired with a bit that is 0)
+                const cd v = t.np == 0 ? t.d[0] : t.d[t.np == 2 ? 3 : 1];
+                if (v != cd(-1.0)) continue;
+                pairs.push_back((double)(a | b << 5));
+                if (pairs.size() == 8) flush();
+            } else if (t.np < 2) {
+                const cd d0 = t.d[0], d1 = t.np ? t.d[1] : t.d[0];
+                raw(RP_PARITY, 0, a, kRpNever, {d0.real(), d0.imag(), d1.real(), d1.imag()});
+            } else {
+                // entry index of the member: 2 x_a + x_b
+                raw(RP_DIAG, 0, a, b, {t.d[0].real(), t.d[0].imag(), t.d[2].real(), t.d[2].imag(),
+                                       t.d[1].real(), t.d[1].imag(), t.d[3].real(), t.d[3].imag()});
+            }
+        }
+        flush();
+    };
+    auto matrix = [&](const Matrix &m) {
+        const uint32_t slot = 1u << (kThreadBits + m.slot);
+        const int c = m.ctl >= 0 ? position_of(m.ctl) : kNone;
+        if (layers.empty()) layers.emplace_back();
+        if (m.real) {
+            if (layers.back().real[m.slot] || (layers.back().raw_uses & slot)) layers.emplace_back();
+            Layer &l = layers.back();
+            l.real[m.slot] = &m;
+            return;
+        }
+        Layer &l = layers.back();
+        l.members++;
+        l.raw.insert(l.raw.end(), m.code, m.code + m.len);
+        l.raw_uses |= slot;
+        if (c >= kThreadBits) l.raw_uses |= 1u << c;
+        if (!m.exchange) return;
+        if (c == kOn) p.sigma[m.slot].one = !p.sigma[m.slot].one;
+        else if (c >= 0 && c < kThreadBits) p.sigma[m.slot].bits ^= 1u << c;
+    };
+    for (int time = 0; time <= last; time++) {
+        if (time & 1) {
+            for (const auto &o : p.order)
+                if (o.first && p.mats[o.second].at == time) matrix(p.mats[o.second]);
+            continue;
+        }
+        std::vector<Table> tabs;
+        Table uniform;  // terms that no slot chooses
+        std::vector<int> alone, free_terms;
+        bool signs_only = true;
+        for (const Term &t : p.terms) signs_only = signs_only && !(t.at == time && !t.sign);
+        for (size_t i = 0; i < p.terms.size(); i++) {
+            const Term &t = p.terms[i];
+            if (t.at != time) continue;
+            if (signs_only) {  // a sign costs less than a table's complex multiply
+                alone.push_back((int)i);
+                continue;
+            }
+            if ((t.mask() & kSlotMask) == 0) {
+                free_terms.push_back((int)i);
+                continue;
+            }
+            uint32_t need = t.mask() & ((1u << kThreadBits) - 1u);
+            for (int k = 0; k < t.np; k++)
+                if (t.pos[k] >= kThreadBits) need |= p.sigma[t.pos[k] - kThreadBits].bits;
+            if (__builtin_popcount(need) > kRpMaxClassBits) {
+                alone.push_back((int)i);
+                continue;
+            }
+            Table *to = nullptr;
+            for (Table &tb : tabs)
+                if (!to && __builtin_popcount(tb.bits | need) <= kRpMaxClassBits) to = &tb;
+            if (!to) {
+                tabs.emplace_back();
+                to = &tabs.back();
+            }
+            to->bits |= need;
+            to->terms.push_back((int)i);
+        }
+        // factors without a register position: in a table that has room for their bits
+        for (int i : free_terms) {
+            Table *to = &uniform;
+            for (Table &tb : tabs)
+                if (to == &uniform && __builtin_popcount(tb.bits | p.terms[i].mask()) <= kRpMaxClassBits) to = &tb;
+            to->bits |= p.terms[i].mask();
+            to->terms.push_back(i);
+        }
+        for (const Table &tb : tabs) {
+            Layer l;
+            l.table = (int)table_at.size();
+            for (int i = 0; i < kThreadBits; i++)
+                if ((tb.bits >> i) & 1u) l.class_pos |= (uint32_t)i << (4 * l.class_bits++);
+            layers.push_back(std::move(l));
+            table_at.push_back(tables.size());
+            double fix = 0.0;
+            if (drift && std::fabs(account.open) < kMaxDriftFix)
+                fix = std::min(std::max(account.fixed - account.open, -kMaxDriftFix), kMaxDriftFix) - account.fixed;
+            const auto sums = emit_table(p, tb, std::exp(fix), tables);
+            account.fixed += fix;
+            account.open += fix;
+            if (sums.first > 0.0) account.open += 0.5 * std::log1p((sums.second - sums.first) / sums.first);
+        }
+        if (!uniform.terms.empty()) {
+            double lo = 0.0, hi = 0.0;
+            int nb = 0;
+            for (int i = 0; i < kThreadBits; i++)
+                if ((uniform.bits >> i) & 1u) {
+                    (nb < 4 ? lo : hi) += (double)(i << (4 * (nb & 3)));
+                    nb++;
+                }
+            raw(RP_DIAG, 1, nb, 0, {(double)table_at.size(), lo, hi});
+            table_at.push_back(tables.size());
+            emit_thread_table(p, uniform, tables);
+        }
+        raw_terms(alone);
+    }
+    if (table_at.empty()) return false;
+    // lay out: layer count, layers, tables
+    size_t size = 4;
+    for (Layer &l : layers) {
+        while (l.raw.size() % 4) l.raw.push_back(0.0);
+        size += 4 + l.raw.size();
+        for (const Matrix *m : l.real) size += m ? 8 : 0;
+    }
+    const size_t pad = (4 - out.size() % 4) % 4;
+    if (pad + size + tables.size() > max_reals || layers.size() > 1000) return false;
+    out.resize(out.size() + pad, 0.0);
+    res = ph;
+    res.mat = (int32_t)out.size();
+    res.nmat = (int32_t)(size + tables.size());
+    out.insert(out.end(), {(double)layers.size(), 0.0, 0.0, 0.0});
+    for (Layer &l : layers) {
+        uint32_t mask = 0;
+        for (int j = 0; j < kRpBits; j++) mask |= l.real[j] ? 1u << j : 0u;
+        out.push_back((double)(mask | (uint32_t)l.class_bits << 10 | (l.table >= 0 ? 1u << 13 : 0u)));
+        out.push_back(l.table >= 0 ? (double)(size + table_at[(size_t)l.table]) : 0.0);
+        out.push_back((double)l.class_pos);
+        out.push_back((double)(l.members | (uint32_t)(l.raw.size() / 4) << 8));
+        for (const Matrix *m : l.real)
+            if (m) out.insert(out.end(), {m->code[1], m->code[2], m->code[3], m->code[4],   // M
+                                          m->code[4], m->code[3], m->code[2], m->code[1]}); // X M X
+        // a thread table's member names its table by number until here
+        for (size_t at = 0, k = 0; k < (size_t)l.members; k++) {
+            const int code = (int)l.raw[at];
+            if ((code & 7) == RP_DIAG && ((code >> 3) & 7) == 1)
+                l.raw[at + 1] = (double)(size + table_at[(size_t)l.raw[at + 1]]);
+            at += 1 + ((code >> 16) & 255);
+        }
+        out.insert(out.end(), l.raw.begin(), l.raw.end());
+    }
+    out.insert(out.end(), tables.begin(), tables.end());
+    if (drift) *drift = account;
+    return true;
+}
+
+}  // namespace
+
+std::vector<KOp> pack_register_phases(const std::vector<KOp> &kops, const std::vector<double> &mats, size_t max_reals,
+                                      std::vector<double> &out, RoundingDrift *drift) {
+    std::vector<KOp> res(kops);
+    out.reserve(std::max(max_reals, mats.size() + 16 * kops.size()));
+    size_t left = 0;  // reals of the ops not packed yet, as they are
+    for (const KOp &k : kops) left += (size_t)k.nmat + 16;
+    for (KOp &k : res) {
+        left -= (size_t)k.nmat + 16;
+        KOp packed;
+        if (k.fkind == F_RPHASE && out.size() + left < max_reals &&
+            pack_phase(k, mats, max_reals - out.size() - left, drift, out, packed)) {
+            k = packed;
+            continue;
+        }
+        if (k.fkind == F_RPHASE) {  // its members as they are, in one layer
+            while (out.size() % 4) out.push_back(0.0);
+            const size_t at = out.size(), reals = (size_t)k.nmat - 1, padded = (reals + 3) / 4 * 4;
+            out.insert(out.end(), {1.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0,
+                                   (double)((int)mats[(size_t)k.mat] | (int)(padded / 4) << 8)});
+            out.insert(out.end(), mats.begin() + k.mat + 1, mats.begin() + k.mat + k.nmat);
+            out.resize(at + 8 + padded, 0.0);
+            k.mat = (int32_t)at;
+            k.nmat = (int32_t)(8 + padded);
+            continue;
+        }
+        const int at = (int)out.size();
+        out.insert(out.end(), mats.begin() + k.mat, mats.begin() + k.mat + k.nmat);
+        k.mat = at;
+    }
+    return res;
+}
+
+}  // namespace qs

@@ -232,13 +232,15 @@ __device__ __forceinline__ void dense_k_smem(typename C2T<T>::type *tile, const 
 // Program (floats, staged in shared memory): member count, then per member a code and
 // `len` payload reals.  code = type | slot << 3 | a << 6 | b << 11 | len << 16, where a
 // and b name positions: 16 + slot for a register position, the thread-index bit for any
-// other, kRpAlways / kRpNever for a bit that is 1 / 0 for every amplitude.
+// other, kRpAlways / kRpNever for a bit that is 1 / 0 for every amplitude.  Passes of many tiles
+// run programs in layers instead (kops.cuh): a factor table for all diagonals between two
+// layers of matrices, real matrices read together, members for the rest.
 //
 // An exchange (X, or CNOT whose control is not a register position) is not carried out:
 // it toggles bit `slot` of sigma, i.e. relabels which register holds which amplitude, and
 // every later member and the final store read the relabelled order.
 constexpr int kRpRegs = 1 << kRpBits;
-static_assert(kRpMaxMembers * 9 + 1 <= kMaxOpReals, "a phase program must fit the staged reals");
+static_assert(kRpMaxMembers * 9 + 8 <= kMaxOpReals, "a phase program must fit the staged reals");
 
 // Bit r set iff bit j of r is set (j < kRpBits; index 5..7 unused).
 static __constant__ uint32_t c_rp_pattern[8] = {0xAAAAAAAAu, 0xCCCCCCCCu, 0xF0F0F0F0u, 0xFF00FF00u, 0xFFFF0000u, 0u, 0u, 0u};
@@ -305,18 +307,18 @@ __device__ __forceinline__ void rp_m1(float2 (&v)[kRpRegs], const float (&M)[8])
     }
 }
 
-// real 2x2 (a b; c d): 4 multiply-adds per amplitude
+// real 2x2 (a b; c d): 4 multiply-adds per amplitude, on the real and imaginary part at once
+// (the FP32 pipe takes as long, but half the issue slots are left to its other work)
 template <int J>
 __device__ __forceinline__ void rp_mr(float2 (&v)[kRpRegs], float a, float b, float c, float d) {
+    const float2 A = make_float2(a, a), B = make_float2(b, b), C = make_float2(c, c), D = make_float2(d, d);
 #pragma unroll
     for (int r = 0; r < kRpRegs; r++) {
         if (r & (1 << J)) continue;
         float2 &x = v[r], &y = v[r | (1 << J)];
-        const float pxr = b * y.x, pxi = b * y.y, pyr = c * x.x, pyi = c * x.y;
-        x.x = fmaf(a, x.x, pxr);
-        x.y = fmaf(a, x.y, pxi);
-        y.x = fmaf(d, y.x, pyr);
-        y.y = fmaf(d, y.y, pyi);
+        const float2 px = __fmul2_rn(B, y), py = __fmul2_rn(C, x);
+        x = __ffma2_rn(A, x, px);
+        y = __ffma2_rn(D, y, py);
     }
 }
 
@@ -453,6 +455,37 @@ __device__ __forceinline__ void rp_table(float2 (&v)[kRpRegs], const float *tabl
     }
 }
 
+// Class of this thread for a table member: bit i is the thread-index bit named by the i-th 4
+// bits of (lo, hi).
+__device__ __forceinline__ uint32_t rp_class(uint32_t lo, uint32_t hi, int nb, uint32_t tid) {
+    uint32_t c = 0;
+    for (int i = 0; i < nb; i++) {
+        c |= ((tid >> (lo & 15u)) & 1u) << i;
+        lo = (lo >> 4) | (i == 3 ? hi : 0u);
+    }
+    return c;
+}
+
+// multiply register r by its class's factor: 16 loads of 16 bytes, one complex multiply each;
+// STEP: 16-byte units between a class's loads (0: `step`)
+template <int STEP>
+__device__ __forceinline__ void rp_class_table(float2 (&v)[kRpRegs], const float4 *p, uint32_t step) {
+#pragma unroll
+    for (int k = 0; k < kRpRegs / 2; k++) {
+        const float4 t = STEP ? p[k * STEP] : *p;
+        if (!STEP) p += step;
+        v[2 * k] = rp_cmul(v[2 * k], t.x, t.y);
+        v[2 * k + 1] = rp_cmul(v[2 * k + 1], t.z, t.w);
+    }
+}
+
+// a layer's real matrix on slot J; X M X (the second 4 reals) in lanes whose bit of sigma is set
+template <int J>
+__device__ __forceinline__ void rp_layer_real(float2 (&v)[kRpRegs], const float4 *P, uint32_t sigma) {
+    const float4 q = P[(sigma >> J) & 1u];
+    rp_mr<J>(v, q.x, q.y, q.z, q.w);
+}
+
 __device__ __forceinline__ void rp_ph(float2 (&v)[kRpRegs], float pr, float pi, uint32_t K) {
     if (K == 0u) return;
     if (K == 0xFFFFFFFFu) {
@@ -539,33 +572,29 @@ __device__ __forceinline__ void rp_phase_run(float2 (&v)[kRpRegs], const float *
     }
 }
 
-// Tile index of register 0 of this thread (register r: base ^ XOR of pb[j] over the bits
-// j of r), sigma and the per-slot position bits of phase ph.
+// Byte offset in the tile of register 0 of this thread (register r: base ^ XOR of pb[j] over
+// the bits j of r), sigma and the byte offsets of the slot positions of phase ph.  The thread
+// index's bits go to the positions that are not slots, in order: a zero bit is opened at each
+// slot's position in turn.  The slots of positions below 4 are the lowest ones, so sigma is a
+// field of the lane index.
 __device__ __forceinline__ void rp_geometry(const KOp &ph, uint32_t tid, uint32_t (&pb)[kRpBits], uint32_t &base,
                                             uint32_t &sigma) {
-    const uint32_t lane = tid & 31u;
     int nlow = 0;
+    base = tid;
 #pragma unroll
     for (int j = 0; j < kRpBits; j++) {
-        pb[j] = 1u << ph.pos[j];
+        pb[j] = 8u << ph.pos[j];
         nlow += ph.pos[j] < 4 ? 1 : 0;
+        base += base & (0u - (1u << ph.pos[j]));
     }
-    sigma = 0;
-    int li = 4 - nlow;
+    sigma = ((tid & 15u) >> (4 - nlow)) & ((1u << nlow) - 1u);
+    base *= 8u;
 #pragma unroll
-    for (int j = 0; j < kRpBits; j++)
-        if (ph.pos[j] < 4) {
-            sigma |= ((lane >> li) & 1u) << j;
-            li++;
-        }
-    base = 0;
-    for (int i = 0; i < ph.nt; i++) base |= ((tid >> i) & 1u) << (uint32_t)((ph.off[0] >> (4 * i)) & 15u);
-#pragma unroll
-    for (int j = 0; j < kRpBits; j++) base ^= ((sigma >> j) & 1u) ? pb[j] : 0u;
+    for (int j = 0; j < 4; j++) base ^= ((sigma >> j) & 1u) ? pb[j] : 0u;
 }
 
 template <int R>
-__device__ __forceinline__ uint32_t rp_index(uint32_t base, const uint32_t (&pb)[kRpBits]) {
+__device__ __forceinline__ uint32_t rp_offset(uint32_t base, const uint32_t (&pb)[kRpBits]) {
     uint32_t o = base;
 #pragma unroll
     for (int j = 0; j < kRpBits; j++)
@@ -577,7 +606,7 @@ template <int R>
 __device__ __forceinline__ void rp_load(float2 (&v)[kRpRegs], const float2 *tile, uint32_t base,
                                         const uint32_t (&pb)[kRpBits]) {
     if constexpr (R < kRpRegs) {
-        v[R] = tile[rp_index<R>(base, pb)];
+        v[R] = *(const float2 *)((const char *)tile + rp_offset<R>(base, pb));
         rp_load<R + 1>(v, tile, base, pb);
     }
 }
@@ -585,12 +614,22 @@ template <int R>
 __device__ __forceinline__ void rp_store(const float2 (&v)[kRpRegs], float2 *tile, uint32_t base,
                                          const uint32_t (&pb)[kRpBits]) {
     if constexpr (R < kRpRegs) {
-        tile[rp_index<R>(base, pb)] = v[R];
+        *(float2 *)((char *)tile + rp_offset<R>(base, pb)) = v[R];
         rp_store<R + 1>(v, tile, base, pb);
     }
 }
 
-// Runs one phase: every thread of the block must call this.
+// Runs one phase: every thread of the block must call this.  Bound: the FP32 pipe and
+// instruction issue (a brickwork pass of 26 qubits: FMA pipe 44 %, issue 56 %, HBM 18 %; the
+// rest is dependency latency at 4 warps per scheduler, the registers of 32 amplitudes).  So a
+// phase is made of few instructions: real 2x2 matrices in packed FP32 (64 per warp and gate),
+// one complex multiply and half a load per amplitude for all diagonals between two layers of
+// matrices, one read of the program per layer.  28-qubit brickwork of 40 layers 117.5 -> 67.0 ms
+// (74.4 ms before offsets in bytes and run offsets made once), 30-qubit QAOA p = 4 99.6 -> 71.6
+// ms, 25-qubit Trotter circuit of 16 steps 7.4 -> 5.0 ms.  LAYERS: the program is in layers
+// (passes of many tiles); else it is a member count and the members.  Two instances, since
+// reading both in one cost the plain form 12 % (small states wait for single tiles).
+template <bool LAYERS>
 __device__ __forceinline__ void rphase_run(float2 *tile, const KOp &ph, const float *prog) {
     const uint32_t tid = threadIdx.x;
     float2 v[kRpRegs];
@@ -600,14 +639,38 @@ __device__ __forceinline__ void rphase_run(float2 *tile, const KOp &ph, const fl
         rp_geometry(ph, tid, pb, base, sigma);
         rp_load<0>(v, tile, base, pb);
     }
-    const int nmem = (int)rp_int(prog[0]);
-    const float *mm = prog + 1;
-    for (int i = 0; i < nmem; i++) {
+    // at: the next real of the program; layers and members left to do, counted in one register
+    uint32_t at = LAYERS ? 4u : 1u, left = rp_int(prog[0]) << (LAYERS ? 8 : 0);
+    while (left) {
+        if (LAYERS && !(left & 255u)) {  // the next layer's table and real matrices
+            const float4 *P = (const float4 *)(prog + at);
+            const float4 h = *P++;
+            const uint32_t h0 = rp_int(h.x);
+            if (h0 & (1u << 13)) {
+                const int nb = (int)((h0 >> 10) & 7u);
+                const float4 *table = (const float4 *)(prog + rp_int(h.y));
+                if (nb == 0) rp_class_table<1>(v, table, 1u);
+                else if (nb == 1) rp_class_table<2>(v, table + ((tid >> rp_int(h.z)) & 1u), 2u);
+                else rp_class_table<0>(v, table + rp_class(rp_int(h.z), 0u, nb, tid), 1u << nb);
+            }
+            const float4 *const P0 = P;
+            if (h0 & 1u) { rp_layer_real<0>(v, P, sigma); P += 2; }
+            if (h0 & 2u) { rp_layer_real<1>(v, P, sigma); P += 2; }
+            if (h0 & 4u) { rp_layer_real<2>(v, P, sigma); P += 2; }
+            if (h0 & 8u) { rp_layer_real<3>(v, P, sigma); P += 2; }
+            if (h0 & 16u) { rp_layer_real<4>(v, P, sigma); P += 2; }
+            left += (rp_int(((const float *)P0)[-1]) & 255u) - 256u;
+            at = (uint32_t)((const float *)P - prog);
+            continue;
+        }
+        left--;
+        const float *mm = prog + at;
         const int code = (int)rp_int(mm[0]);
         const int type = code & 7, J = (code >> 3) & 7, ea = (code >> 6) & 31, eb = (code >> 11) & 31;
         const int len = (code >> 16) & 255;
         const float *P = mm + 1;
-        mm += 1 + len;
+        at += 1u + (uint32_t)len;
+        if (LAYERS && !(left & 255u)) at = (at + 3u) & ~3u;  // layers start at multiples of 4 reals
         switch (type) {
         case RP_M1:
             if (eb == RP_R0) {
@@ -689,6 +752,11 @@ __device__ __forceinline__ void rphase_run(float2 *tile, const KOp &ph, const fl
             break;
         }
         case RP_DIAG: {
+            if (LAYERS && J != 0) {  // one factor per thread, from a table
+                const float *f = prog + rp_int(P[0]) + 2 * rp_class(rp_int(P[1]), rp_int(P[2]), ea, tid);
+                rp_scale(v, f[0], f[1]);
+                break;
+            }
             float M[8];
 #pragma unroll
             for (int e = 0; e < 8; e++) M[e] = P[e];
@@ -748,8 +816,8 @@ __device__ __forceinline__ void rphase_run(float2 *tile, const KOp &ph, const fl
 
 // Applies one op to the tile; op and its matrix entries are in shared memory.  RP = false
 // leaves the register-phase code out (kernels that never receive F_RPHASE ops keep their
-// registers for themselves).
-template <typename T, bool RP = true, bool IX = false>
+// registers for themselves); LAYERS: register phases are in layers (pack_register_phases).
+template <typename T, bool RP = true, bool IX = false, bool LAYERS = false>
 __device__ __forceinline__ void apply_op_smem(typename C2T<T>::type *tile, const KOp &op, const T *sm, int m) {
     if constexpr (IX && std::is_same<T, double>::value) {
         // complex128 integer products (QS_PREC_IX64) for one-qubit dense ops and diagonal ops
@@ -839,7 +907,7 @@ __device__ __forceinline__ void apply_op_smem(typename C2T<T>::type *tile, const
         else if (op.k == 4) dense_k_smem<T, 4>(tile, op, sm, m);
         break;
     case F_RPHASE:
-        if constexpr (std::is_same<T, float>::value && RP) rphase_run(tile, op, sm);
+        if constexpr (std::is_same<T, float>::value && RP) rphase_run<LAYERS>(tile, op, sm);
         break;
     default:
         break;

@@ -323,3 +323,18 @@ def test_register_phases_phase_layers(qs, n):
     got, st = _run_c64(qs, n, psi0, gates)
     assert np.max(np.abs(got - want)) <= TOL_C64
     assert fidelity_gap(got, want) <= 1e-6
+
+
+@pytest.mark.parametrize("n", [21, 22, 23])
+def test_register_phases_in_layers(qs, n):
+    """complex64 passes of 2^9 tiles and more (22 qubits; 21 stays plain) run their phases in
+    layers of factor tables and real matrices: every gate type a phase holds, with exchanges that
+    relabel registers, controls in and outside the register positions, diagonals on all of them
+    and equal angles repeated, against the oracle."""
+    gates = inputs.random_circuit(n, 250, seed=60 + n) + inputs.brickwork(n, 4, seed=n) + inputs.tfim(n, 3) + \
+        inputs.qaoa_3regular(n, p=1, seed=n) + inputs.random_circuit(n, 60, seed=n)
+    psi0 = inputs.gaussian_state(n, seed=n).astype(np.complex64)
+    want = oracle.run(psi0.astype(np.complex128), n, gates)
+    got, _ = _run_c64(qs, n, psi0, gates)
+    assert np.max(np.abs(got - want)) <= TOL_C64
+    assert fidelity_gap(got, want) <= 1e-6
