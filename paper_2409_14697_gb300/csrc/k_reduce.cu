@@ -8,14 +8,17 @@
 //    records, adding the 8 qubits spelled by the record index within the group; the last
 //    level combines the few second-level records.  Everything is summed in a fixed order
 //    (per-thread pairwise trees, fixed butterfly trees, fixed upper levels), so results
-//    are bitwise reproducible whatever else runs on the GPU.  complex128 sums in FP64;
-//    complex64 sums each thread's groups of 16 exact squares in double-float FP32 and
-//    everything above in FP64 (FP64 throughput is the limit of these passes on GB300).
+//    are bitwise reproducible whatever else runs on the GPU.  complex128 sums each
+//    thread's groups of 16 |a|^2 in 64-bit integers, complex64 its groups of 32 exact
+//    squares in double-float FP32, and both everything above in FP64 (at 2 FP64
+//    instructions per clock and SM the squares alone would take longer than the read).
 //  * top-K |a|^2: exact radix select of the K-th largest key (the bit pattern of the
 //    non-negative probability, monotone in its value), then a deterministic gather of
 //    the elements above it and of the lowest-index ties, then one-block bitonic sort.
 //  * |0...0> and scaling.
 #include <algorithm>
+#include <cmath>
+#include <cstring>
 #include <mutex>
 #include <type_traits>
 
@@ -42,7 +45,9 @@ __device__ __forceinline__ double f2d_exact(float x) {
     return __hiloint2double((int)hi, (int)((b & 7u) << 29));
 }
 // Sums of |a|^2 inside one thread of the first level, over a group of 16 or 32 amplitudes.
-// complex128: FP64, with a pair of amplitudes summed as one chain of fused multiply-adds.
+// complex128: 64-bit integers relative to the group's largest magnitude (SumU64); groups whose
+// exponents are out of that form's range in FP64, with a pair of amplitudes summed as one chain
+// of fused multiply-adds (SumF64).
 // complex64: the squares of the stored floats are exact as FP32 pairs (x*x and
 // fma(x, x, -x*x)) and are added as double-float values (hi, lo: an FP32 two-sum per
 // addition, then a renormalisation), so a group's sums run on the FP32 pipe and the FP64
@@ -60,6 +65,35 @@ struct SumF64 {
         return __fma_rn(a.x, a.x, __fma_rn(a.y, a.y, pb));
     }
     static __device__ __forceinline__ double to_double(T a) { return a; }
+};
+// Sums of squares as integers.  E: the biased exponent of the group's largest |x|.  A real x of
+// the group becomes X = floor(|x| 2^(1083 - E)) < 2^61 (its significand shifted right by E - e),
+// its square the top 64 bits of X^2, short of the exact value by less than 6 units of
+// 2^(2 E - 2102) (3 from the shifted X, 3 from the low words), 2^-56 of the largest square at most 6
+// times.  A group's sum of up to 32 squares is below 2^63 and exact beyond that, so it is
+// within 32 * 6 units of its exact value, 2^-50.4 of its largest square and, as the units lost
+// are those of the many terms that make the sum large, about 2^-54 of a sum of comparable
+// terms: the rounding of a FP64 chain.  One integer-to-double conversion per group sum.
+// 20 integer instructions per real against 1.25-1.75 FP64 instructions (16 times slower each).
+struct SumU64 {
+    using T = unsigned long long;
+    static constexpr uint32_t kMinExp = 560, kMaxExp = 1500;  // group sums and masses stay normal doubles
+    static __device__ __forceinline__ T add(T a, T b) { return a + b; }
+    static __device__ __forceinline__ T square(double x, uint32_t E) {
+        const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+        const uint32_t e = (hi >> 20) & 0x7FFu;
+        const uint32_t mh = (hi & 0xFFFFFu) | 0x100000u;
+        // M 2^8, then right by E - e (PTX clamps shifts to 64: e = 0, a zero or subnormal, gives 0)
+        unsigned long long X = ((unsigned long long)__funnelshift_l(lo, mh, 8) << 32) | (lo << 8);
+        asm("shr.b64 %0, %0, %1;" : "+l"(X) : "r"(E - e));
+        const uint32_t xh = (uint32_t)(X >> 32), xl = (uint32_t)X;
+        return (unsigned long long)xh * xh + 2ull * __umulhi(xh, xl);
+    }
+    static __device__ __forceinline__ T leaf(double2 a, uint32_t E) { return square(a.x, E) + square(a.y, E); }
+    static __device__ __forceinline__ double to_double(T a, uint32_t E) {
+        const double d = __ull2double_rn(a);
+        return a ? __hiloint2double(__double2hiint(d) + (int)((2u * E - 2102u) << 20), __double2loint(d)) : 0.0;
+    }
 };
 struct SumDF32 {
     using T = float2;  // (hi, lo), |lo| <= ulp(hi) / 2
@@ -89,10 +123,6 @@ struct SumDF32 {
     // hi + lo spans at most 48 significant bits: the FP64 sum is exact
     static __device__ __forceinline__ double to_double(T a) { return __dadd_rn(f2d_exact(a.x), f2d_exact(a.y)); }
 };
-template <typename V> struct SumOf;
-template <> struct SumOf<double2> { using S = SumF64; };
-template <> struct SumOf<float2> { using S = SumDF32; };
-
 
 // Butterfly sum over a warp: fixed order, identical result in every lane.
 __device__ __forceinline__ double warp_sum(double v) {
@@ -130,6 +160,62 @@ struct TreeLevels {
     }
 };
 
+// Total and masses of the U low loop bits of a group of 2^U amplitudes, as doubles.
+template <int U, int BITS, typename S, typename V>
+__device__ __forceinline__ void group_tree(const V *v, double &gd, double *md) {
+    using A = typename S::T;
+    if constexpr (U == 0) {
+        gd = S::to_double(S::leaf(v[0]));
+    } else {
+        constexpr int H = 1 << (U - 1);  // pairs
+        A cur[H], odd[H], mass[U];
+#pragma unroll
+        for (int i = 0; i < H; i++) cur[i] = S::pair(v[2 * i], v[2 * i + 1], odd[i]);
+        if (BITS) mass[0] = tree_sum<S, H>(odd);
+        gd = S::to_double(TreeLevels<S, 1, H, BITS>::run(cur, mass));
+        if (BITS)
+#pragma unroll
+            for (int l = 0; l < U; l++) md[l] = S::to_double(mass[l]);
+    }
+}
+template <int U, int BITS>
+__device__ __forceinline__ void group_sums(const float2 *v, double &gd, double *md) {
+    group_tree<U, BITS, SumDF32>(v, gd, md);
+}
+template <int U, int BITS>
+__device__ __forceinline__ void group_sums(const double2 *v, double &gd, double *md) {
+    using S = SumU64;
+    constexpr int N = 1 << U, H = U > 0 ? (1 << (U - 1)) : 1;
+    uint32_t top = 0;  // high word of the largest magnitude
+#pragma unroll
+    for (int i = 0; i < N; i++)
+        top = max(top, max((uint32_t)__double2hiint(v[i].x) & 0x7FFFFFFFu, (uint32_t)__double2hiint(v[i].y) & 0x7FFFFFFFu));
+    const uint32_t E = top >> 20;
+    if (E - S::kMinExp <= S::kMaxExp - S::kMinExp) {
+        S::T cur[H], odd[H], mass[U > 0 ? U : 1];
+        if constexpr (U == 0) {
+            cur[0] = S::leaf(v[0], E);
+        } else {
+#pragma unroll
+            for (int i = 0; i < H; i++) {
+                odd[i] = S::leaf(v[2 * i + 1], E);
+                cur[i] = S::leaf(v[2 * i], E) + odd[i];
+            }
+            if (BITS) mass[0] = tree_sum<S, H>(odd);
+        }
+        gd = S::to_double(TreeLevels<S, 1, H, BITS>::run(cur, mass), E);
+        if (BITS)
+#pragma unroll
+            for (int l = 0; l < U; l++) md[l] = S::to_double(mass[l], E);
+    } else if (E == 0) {  // zeros and subnormals: their squares are 0
+        gd = 0.0;
+#pragma unroll
+        for (int l = 0; l < U; l++) md[l] = 0.0;
+    } else {
+        group_tree<U, BITS, SumF64>(v, gd, md);
+    }
+}
+
 // Level 1: part[blk*(cb+1) + 0] = block total; part[blk*(cb+1) + 1 + q] = mass with bit q
 // set, q < cb.  JB = loop bits per thread (cb = tb + JB); BITS = 0: totals only (the same
 // operations in the same order, so a norm equals the total of a <Z_q> call bit for bit).
@@ -141,12 +227,9 @@ struct TreeLevels {
 template <typename V, int JB, int BITS>
 __global__ void __launch_bounds__(256)
 k_expz_part(const V *__restrict__ psi, int cb, int tb, double *__restrict__ part) {
-    using S = typename SumOf<V>::S;
-    using A = typename S::T;
     constexpr int UMAX = std::is_same<V, float2>::value ? 5 : 4;
     constexpr int U = JB < UMAX ? JB : UMAX;
     constexpr int NJ = JB > 0 ? JB : 1;
-    constexpr int H = U > 0 ? (1 << (U - 1)) : 1;  // pairs per group
     __shared__ double s_tot[256];
     __shared__ double s_j[NJ][256];
     const int T = 1 << tb, t = threadIdx.x;
@@ -159,21 +242,12 @@ k_expz_part(const V *__restrict__ psi, int cb, int tb, double *__restrict__ part
         V v[1 << U];
 #pragma unroll
         for (int j = 0; j < (1 << U); j++) v[j] = psi[start + ((uint64_t)((g << U) + j) << tb) + t];
-        A gt, mass[U > 0 ? U : 1];
-        if constexpr (U == 0) {
-            gt = S::leaf(v[0]);
-        } else {
-            A cur[H], odd[H];
-#pragma unroll
-            for (int i = 0; i < H; i++) cur[i] = S::pair(v[2 * i], v[2 * i + 1], odd[i]);
-            if (BITS) mass[0] = tree_sum<S, H>(odd);
-            gt = TreeLevels<S, 1, H, BITS>::run(cur, mass);
-        }
-        const double gd = S::to_double(gt);
+        double gd, md[U > 0 ? U : 1];
+        group_sums<U, BITS>(v, gd, md);
         tot = __dadd_rn(tot, gd);
         if (BITS) {
 #pragma unroll
-            for (int l = 0; l < U; l++) jacc[l] = __dadd_rn(jacc[l], S::to_double(mass[l]));
+            for (int l = 0; l < U; l++) jacc[l] = __dadd_rn(jacc[l], md[l]);
 #pragma unroll
             for (int b = U; b < JB; b++)
                 if ((g >> (b - U)) & 1) jacc[b] = __dadd_rn(jacc[b], gd);
