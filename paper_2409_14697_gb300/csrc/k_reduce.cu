@@ -12,7 +12,8 @@
 //    thread's groups of 16 |a|^2 in 64-bit integers, complex64 its groups of 32 exact
 //    squares in double-float FP32, and both everything above in FP64 (at 2 FP64
 //    instructions per clock and SM the squares alone would take longer than the read).
-//  * top-K |a|^2: exact radix select of the K-th largest key (the bit pattern of the
+//  * top-K |a|^2: an FP32 prefilter above a sampled or counted threshold with exact keys for the
+//    candidates; where they do not fit, exact radix select of the K-th largest key (the bit pattern of the
 //    non-negative probability, monotone in its value), then a deterministic gather of
 //    the elements above it and of the lowest-index ties, then one-block bitonic sort.
 //  * |0...0> and scaling.
@@ -560,7 +561,10 @@ k_topk_sort(const V *__restrict__ psi, const unsigned long long *key, const unsi
     if ((*skip != 0) == (skip_when != 0)) return;
     extern __shared__ unsigned long long sm[];
     unsigned long long *sk = sm, *si = sm + P;
-    if (n_in < 0) n_in = (int)min(*n_in_dev, (unsigned int)P);  // candidate count (fast path)
+    if (n_in < 0) {  // candidate count (fast path): sort no more than it takes
+        n_in = (int)min(*n_in_dev, (unsigned int)P);
+        while (P / 2 >= n_in && P / 2 >= K) P >>= 1;
+    }
     for (int i = threadIdx.x; i < P; i += blockDim.x) {
         sk[i] = i < n_in ? key[i] : 0ull;
         si[i] = i < n_in ? idx[i] : ~0ull;
@@ -603,13 +607,36 @@ k_topk_sort(const V *__restrict__ psi, const unsigned long long *key, const unsi
 // exact selection and tie order.
 constexpr int kTkBins = 2048;
 constexpr int kTkCap = 8192;  // candidates the one-block sort holds
+constexpr uint64_t kTkSampleBytes = 64ull << 20;  // smallest state whose threshold is sampled
 
+// One read: the threshold is first estimated from a sample (one 128-byte line of every 64 or
+// 32, at a place that a hash chooses), so that about K + 4.5 standard deviations of it are
+// expected above; the state is then read once for everything above it.  That selection holds
+// the exact top K if it fits the sort and at least K of it lie a fine bin above the threshold;
+// otherwise the three-read form below runs.  Bound: the one read of the state (28 qubits
+// complex128, with norm and <Z_q>: 3.87 -> 2.22 ms; at 11 qubits, where launches are the time, 491
+// -> 138 us: a call that waits launches the next selection only where one was not complete).
 struct TkState {
-    int ok;                  // 1: fast path chosen (the exact pipeline then returns at once)
+    int ok;                  // 1: candidates are complete (the exact pipeline then returns at once)
     unsigned int cnt;        // candidates collected (must follow ok)
     unsigned int b1, thr;    // coarse bin of the K-th value, threshold on bits >> 9
     unsigned long long above1, need1;
+    int sampled;             // 1: a sampled threshold is in thr
+    unsigned int cnt_above;  // candidates at fine bin thr + 1 or above
+    int done;                // 1: the sampled selection is complete
 };
+
+// Sample of one line of 128 bytes in every 2^sb: element of sample slot i.
+template <typename V>
+__device__ __forceinline__ uint64_t sample_index(uint64_t i, int sb) {
+    constexpr int LB = sizeof(V) == 16 ? 3 : 4;  // elements per line
+    const uint64_t line = i >> LB;
+    uint32_t h = (uint32_t)line * 0x9E3779B1u ^ (uint32_t)(line >> 32) * 0x85EBCA77u;
+    h ^= h >> 15;
+    h *= 0x2C1B3C6Du;
+    h ^= h >> 13;
+    return (((line << sb) | (h & ((1u << sb) - 1u))) << LB) | (i & ((1u << LB) - 1u));
+}
 
 __device__ __forceinline__ float trunc_f32(double x) {
     const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
@@ -624,16 +651,19 @@ __device__ __forceinline__ uint32_t p32_bits(double2 a) {
 }
 __device__ __forceinline__ uint32_t p32_bits(float2 a) { return __float_as_uint(fmaf(a.x, a.x, a.y * a.y)); }
 
-template <typename V, int LEVEL>
+// SAMPLE: over the n sample slots (one line in 2^sb); else over the state, unless the sampled
+// selection was complete.
+template <typename V, int LEVEL, bool SAMPLE>
 __global__ void __launch_bounds__(256)
-k_tk_hist(const V *__restrict__ psi, uint64_t n, const TkState *__restrict__ ts,
+k_tk_hist(const V *__restrict__ psi, uint64_t n, int sb, const TkState *__restrict__ ts,
           unsigned long long *__restrict__ hist) {
+    if (!SAMPLE && ts->ok) return;
     __shared__ unsigned int h[kTkBins];
     for (int i = threadIdx.x; i < kTkBins; i += 256) h[i] = 0;
     __syncthreads();
     const uint32_t b1 = LEVEL == 2 ? ts->b1 : 0u;
     for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (uint64_t)gridDim.x * 256) {
-        const uint32_t b = p32_bits(psi[i]);
+        const uint32_t b = p32_bits(psi[SAMPLE ? sample_index<V>(i, sb) : i]);
         if (LEVEL == 1) atomicAdd(&h[b >> 20], 1u);
         else if ((b >> 20) == b1) atomicAdd(&h[(b >> 9) & (kTkBins - 1)], 1u);
     }
@@ -642,36 +672,92 @@ k_tk_hist(const V *__restrict__ psi, uint64_t n, const TkState *__restrict__ ts,
         if (h[i]) atomicAdd(&hist[i], (unsigned long long)h[i]);
 }
 
-__global__ void k_tk_plan1(const unsigned long long *__restrict__ h1, unsigned long long K, TkState *ts) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    unsigned long long acc = 0;
-    int b = kTkBins - 1;
-    for (; b > 0; b--) {
-        if (acc + h1[b] >= K) break;
-        acc += h1[b];
+// The highest bin b with at least `need` of hist[b..kTkBins - 1], and the count above it.  One block of 1024 threads, two bins each.
+__device__ __forceinline__ void tk_pick(const unsigned long long *__restrict__ hist, unsigned long long need, int &bin,
+                                        unsigned long long &above) {
+    __shared__ unsigned long long s[1024];
+    __shared__ int s_bin;
+    __shared__ unsigned long long s_above;
+    const int t = threadIdx.x;
+    // thread t holds the bins 2047 - 2t and 2046 - 2t: inclusive sums run from the top
+    const unsigned long long hi = hist[kTkBins - 1 - 2 * t], lo = hist[kTkBins - 2 - 2 * t];
+    s[t] = hi + lo;
+    if (t == 0) {
+        s_bin = 0;
+        s_above = 0;
     }
-    ts->b1 = (unsigned int)b;
-    ts->above1 = acc;
-    ts->need1 = K - acc;
-    ts->ok = 0;
-    ts->cnt = 0;
+    __syncthreads();
+    for (int d = 1; d < 1024; d <<= 1) {
+        const unsigned long long v = t >= d ? s[t - d] : 0ull;
+        __syncthreads();
+        s[t] += v;
+        __syncthreads();
+    }
+    const unsigned long long before = s[t] - hi - lo;
+    if (before < need && before + hi >= need) {
+        s_bin = kTkBins - 1 - 2 * t;
+        s_above = before;
+    } else if (before + hi < need && s[t] >= need) {
+        s_bin = kTkBins - 2 - 2 * t;
+        s_above = before + hi;
+    } else if (t == 1023 && s[t] < need) {  // fewer than need in all: the lowest bin
+        s_bin = 0;
+        s_above = s[t] - lo;
+    }
+    __syncthreads();
+    bin = s_bin;
+    above = s_above;
 }
 
-__global__ void k_tk_plan2(const unsigned long long *__restrict__ h1, const unsigned long long *__restrict__ h2,
-                           uint64_t n, TkState *ts) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const unsigned long long need = ts->need1;
-    unsigned long long acc = 0;
-    int b2 = kTkBins - 1;
-    for (; b2 > 0; b2--) {
-        if (acc + h2[b2] >= need) break;
-        acc += h2[b2];
-    }
+__global__ void __launch_bounds__(1024)
+k_tk_plan1(const unsigned long long *__restrict__ h1, unsigned long long K, TkState *ts, int sample) {
+    if (!sample && ts->ok) return;
+    int b;
+    unsigned long long above;
+    tk_pick(h1, K, b, above);
+    if (threadIdx.x != 0) return;
+    ts->b1 = (unsigned int)b;
+    ts->above1 = above;
+    ts->need1 = K - above;
+    ts->ok = 0;
+    ts->cnt = 0;
+    ts->cnt_above = 0;
+    ts->sampled = 0;
+}
+
+// Sample: the threshold, if it is above 0 and the sample promises a selection that fits.
+__global__ void __launch_bounds__(1024)
+k_tk_sampled(const unsigned long long *__restrict__ h2, int sb, TkState *ts) {
+    int b2;
+    unsigned long long above;
+    tk_pick(h2, ts->need1, b2, above);
+    if (threadIdx.x != 0) return;
+    const uint32_t T = (ts->b1 << 11) | (uint32_t)b2;
+    // samples at or above fine bin T, as a count over the state
+    const unsigned long long expect = (ts->above1 + above + h2[b2]) << sb;
+    ts->thr = T;
+    ts->sampled = T >= 1 && expect <= (unsigned long long)kTkCap ? 1 : 0;
+}
+
+// Sampled selection: complete if it holds the top K (see above); otherwise the counters start
+// again for the three-read form.
+__global__ void k_tk_check(TkState *ts, unsigned int K) {
+    if (!ts->sampled) return;
+    if (ts->cnt <= (unsigned int)kTkCap && ts->cnt_above >= K) ts->ok = ts->done = 1;
+}
+
+__global__ void __launch_bounds__(1024)
+k_tk_plan2(const unsigned long long *__restrict__ h1, const unsigned long long *__restrict__ h2,
+           uint64_t n, TkState *ts) {
+    if (ts->ok) return;  // the sampled selection is complete
+    int b2;
+    unsigned long long above;
+    tk_pick(h2, ts->need1, b2, above);
+    if (threadIdx.x != 0) return;
     const uint32_t b1 = ts->b1, T = (b1 << 11) | (uint32_t)b2;
     unsigned long long c;
     if (b2 >= 1) {
-        c = ts->above1;
-        for (int f = b2 - 1; f < kTkBins; f++) c += h2[f];
+        c = ts->above1 + above + h2[b2] + h2[b2 - 1];
     } else if (b1 >= 1) {
         c = ts->above1 + h1[b1] + h1[b1 - 1];  // bound: part of coarse bin b1 - 1 may join
     } else {
@@ -681,19 +767,30 @@ __global__ void k_tk_plan2(const unsigned long long *__restrict__ h1, const unsi
     ts->ok = c <= (unsigned long long)kTkCap ? 1 : 0;
 }
 
-template <typename V>
+// SAMPLED: the selection above the sampled threshold; else the candidates of the three-read form.
+template <typename V, bool SAMPLED>
 __global__ void __launch_bounds__(256)
 k_tk_collect(const V *__restrict__ psi, uint64_t n, TkState *__restrict__ ts,
              unsigned long long *__restrict__ ckey, unsigned long long *__restrict__ cidx) {
-    if (!ts->ok) return;
+    if (SAMPLED ? !ts->sampled : (ts->done || !ts->ok)) return;
     const uint32_t thr = ts->thr;
-    for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (uint64_t)gridDim.x * 256) {
-        const V a = psi[i];
-        if ((p32_bits(a) >> 9) >= thr) {
-            const unsigned int slot = atomicAdd(&ts->cnt, 1u);
-            if (slot < (unsigned int)kTkCap) {
-                ckey[slot] = key_of(a);
-                cidx[slot] = i;
+    constexpr int UN = 4;  // loads in flight per thread
+    const uint64_t step = (uint64_t)gridDim.x * 256 * UN;
+    for (uint64_t i0 = (uint64_t)blockIdx.x * 256 * UN + threadIdx.x; i0 < n; i0 += step) {
+        V a[UN];
+#pragma unroll
+        for (int u = 0; u < UN; u++)
+            if (i0 + u * 256 < n) a[u] = psi[i0 + u * 256];
+#pragma unroll
+        for (int u = 0; u < UN; u++) {
+            if (i0 + u * 256 >= n) continue;
+            const uint32_t f = p32_bits(a[u]) >> 9;
+            if (f >= thr) {
+                const unsigned int slot = atomicAdd(&ts->cnt, 1u);
+                if (SAMPLED && f > thr) atomicAdd(&ts->cnt_above, 1u);
+                if (slot >= (unsigned int)kTkCap) return;  // too many: not complete
+                ckey[slot] = key_of(a[u]);
+                cidx[slot] = i0 + u * 256;
             }
         }
     }
@@ -822,7 +919,7 @@ void reduce_expz(DeviceState &st, double *norm, double *expz) {
 
 namespace {
 struct TopkLayout {
-    size_t o_sel, o_hist, o_tie, o_gt, o_key, o_idx, o_oidx, o_oamp, o_ts, o_h1, o_h2, o_ckey, o_cidx, total;
+    size_t o_sel, o_hist, o_tie, o_gt, o_key, o_idx, o_oidx, o_oamp, o_ts, o_h1, o_h2, o_s1, o_s2, o_ckey, o_cidx, total;
 };
 TopkLayout topk_layout(int n, uint32_t K) {
     const int cb = std::min(n, 12);
@@ -841,6 +938,8 @@ TopkLayout topk_layout(int n, uint32_t K) {
     L.o_ts = carve(sizeof(TkState));
     L.o_h1 = carve(sizeof(unsigned long long) * kTkBins);
     L.o_h2 = carve(sizeof(unsigned long long) * kTkBins);
+    L.o_s1 = carve(sizeof(unsigned long long) * kTkBins);
+    L.o_s2 = carve(sizeof(unsigned long long) * kTkBins);
     L.o_ckey = carve(sizeof(unsigned long long) * kTkCap);
     L.o_cidx = carve(sizeof(unsigned long long) * kTkCap);
     L.total = off;
@@ -850,11 +949,27 @@ TopkLayout topk_layout(int n, uint32_t K) {
 
 size_t scratch_topk_bytes(int n, uint32_t k) { return topk_layout(n, k).total; }
 
-// Launches the whole top-K pipeline; results to idx_dev / amp_dev (device).  The fast path
-// (two histogram passes, one collection pass, one sort) is enqueued first; the exact radix
-// pipeline follows and each of its kernels returns at once when the fast path was taken
-// (a device flag), so nothing waits on the host.
-void top_k_async(DeviceState &st, uint32_t K, uint64_t *idx_dev, double *amp_dev) {
+namespace {
+// The sample for a top-K: one line in 2^sb, and the rank of the threshold in it, 4.5 standard
+// deviations above what K elements of the state leave in the sample.  False: the state is too
+// small for it.
+bool tk_sample_plan(uint64_t bytes, uint64_t n, uint32_t K, int &sb, unsigned long long &rank) {
+    sb = K <= 2048 ? 6 : 5;
+    const double want = (double)K / (double)(1 << sb);
+    rank = 16;
+    while ((double)rank - 4.5 * std::sqrt((double)rank) < want) rank++;
+    // three reads of a state that stays in L2 take no longer than the sample's extra launches
+    return bytes >= kTkSampleBytes && rank <= (n >> sb) / 4;
+}
+
+enum class TopkSelect { all, sampled, three_reads, exact };
+
+// Launches the top-K pipeline; results to idx_dev / amp_dev (device).  The sampled selection is
+// enqueued first, then the three-read form, then the exact radix pipeline; each kernel returns at
+// once when an earlier selection was complete (device flags), so nothing waits on the host.
+// Other values of `select`: that selection alone (ts->ok says whether one of the first two was
+// complete; the exact one finds it 0).
+void topk_launch(DeviceState &st, uint32_t K, uint64_t *idx_dev, double *amp_dev, TopkSelect select) {
     const int n = st.n;
     const uint64_t N = 1ull << n;
     if (K == 0) return;
@@ -888,19 +1003,42 @@ void top_k_async(DeviceState &st, uint32_t K, uint64_t *idx_dev, double *amp_dev
     TkState *ts = (TkState *)(base + TL.o_ts);
     unsigned long long *h1 = (unsigned long long *)(base + TL.o_h1), *h2 = (unsigned long long *)(base + TL.o_h2);
     unsigned long long *ckey = (unsigned long long *)(base + TL.o_ckey), *cidx = (unsigned long long *)(base + TL.o_cidx);
-    QS_CUDA(cudaMemsetAsync(h1, 0, sizeof(unsigned long long) * kTkBins, st.stream));
-    QS_CUDA(cudaMemsetAsync(h2, 0, sizeof(unsigned long long) * kTkBins, st.stream));
-    if (c128) k_tk_hist<double2, 1><<<grid, 256, 0, st.stream>>>((const double2 *)st.psi, N, ts, h1);
-    else k_tk_hist<float2, 1><<<grid, 256, 0, st.stream>>>((const float2 *)st.psi, N, ts, h1);
-    k_tk_plan1<<<1, 1, 0, st.stream>>>(h1, (unsigned long long)K, ts);
-    if (c128) k_tk_hist<double2, 2><<<grid, 256, 0, st.stream>>>((const double2 *)st.psi, N, ts, h2);
-    else k_tk_hist<float2, 2><<<grid, 256, 0, st.stream>>>((const float2 *)st.psi, N, ts, h2);
-    k_tk_plan2<<<1, 1, 0, st.stream>>>(h1, h2, N, ts);
-    if (c128) k_tk_collect<double2><<<grid, 256, 0, st.stream>>>((const double2 *)st.psi, N, ts, ckey, cidx);
-    else k_tk_collect<float2><<<grid, 256, 0, st.stream>>>((const float2 *)st.psi, N, ts, ckey, cidx);
+    unsigned long long *s1 = (unsigned long long *)(base + TL.o_s1), *s2 = (unsigned long long *)(base + TL.o_s2);
+    const bool all = select == TopkSelect::all;
+    // ts, h1, h2, s1 and s2 lie next to one another
+    if (select != TopkSelect::exact)
+        QS_CUDA(cudaMemsetAsync(base + TL.o_ts, 0, TL.o_s2 + sizeof(unsigned long long) * kTkBins - TL.o_ts, st.stream));
+    auto typed = [&](auto psi) {
+        using V = std::remove_const_t<std::remove_pointer_t<decltype(psi)>>;
+        int sb = 0;
+        unsigned long long rank = 0;
+        if ((all || select == TopkSelect::sampled) && tk_sample_plan(N * sizeof(V), N, K, sb, rank)) {
+            const uint64_t ns = N >> sb;
+            const int sgrid = (int)std::min<uint64_t>((ns + 255) / 256, (uint64_t)device_sm_count() * 8);
+            k_tk_hist<V, 1, true><<<sgrid, 256, 0, st.stream>>>(psi, ns, sb, ts, s1);
+            k_tk_plan1<<<1, 1024, 0, st.stream>>>(s1, rank, ts, 1);
+            k_tk_hist<V, 2, true><<<sgrid, 256, 0, st.stream>>>(psi, ns, sb, ts, s2);
+            k_tk_sampled<<<1, 1024, 0, st.stream>>>(s2, sb, ts);
+            k_tk_collect<V, true><<<grid, 256, 0, st.stream>>>(psi, N, ts, ckey, cidx);
+            k_tk_check<<<1, 1, 0, st.stream>>>(ts, K);
+            count_launch(6);
+        }
+        if (!all && select != TopkSelect::three_reads) return;
+        k_tk_hist<V, 1, false><<<grid, 256, 0, st.stream>>>(psi, N, 0, ts, h1);
+        k_tk_plan1<<<1, 1024, 0, st.stream>>>(h1, (unsigned long long)K, ts, 0);
+        k_tk_hist<V, 2, false><<<grid, 256, 0, st.stream>>>(psi, N, 0, ts, h2);
+        k_tk_plan2<<<1, 1024, 0, st.stream>>>(h1, h2, N, ts);
+        k_tk_collect<V, false><<<grid, 256, 0, st.stream>>>(psi, N, ts, ckey, cidx);
+        count_launch(5);
+    };
+    if (c128) typed((const double2 *)st.psi);
+    else typed((const float2 *)st.psi);
     QS_CUDA(cudaGetLastError());
-    sort_launch(ckey, cidx, kTkCap, -1, &ts->cnt, &ts->ok, 0);
-    count_launch(6);
+    if (select != TopkSelect::exact) {
+        sort_launch(ckey, cidx, kTkCap, -1, &ts->cnt, &ts->ok, 0);
+        count_launch();
+    }
+    if (!all && select != TopkSelect::exact) return;
     // ---- exact radix pipeline (returns at once when ts->ok)
     const int *skip = &ts->ok;
     SelState *sel = (SelState *)(base + TL.o_sel);
@@ -938,6 +1076,12 @@ void top_k_async(DeviceState &st, uint32_t K, uint64_t *idx_dev, double *amp_dev
     count_launch(4);
 }
 
+}  // namespace
+
+void top_k_async(DeviceState &st, uint32_t K, uint64_t *idx_dev, double *amp_dev) {
+    topk_launch(st, K, idx_dev, amp_dev, TopkSelect::all);
+}
+
 void top_k(DeviceState &st, uint32_t K, uint64_t *idx, double *amp) {
     if (K == 0) return;
     if ((uint64_t)K > (1ull << st.n) || K > 4096) fail(QS_ERR_INVALID, "top-k: k exceeds min(2^n, 4096)");
@@ -946,10 +1090,23 @@ void top_k(DeviceState &st, uint32_t K, uint64_t *idx, double *amp) {
     char *base = (char *)st.scratch;
     uint64_t *oidx = (uint64_t *)(base + TL.o_oidx);
     double *oamp = (double *)(base + TL.o_oamp);
-    top_k_async(st, K, oidx, oamp);
-    QS_CUDA(cudaMemcpyAsync(idx, oidx, sizeof(uint64_t) * K, cudaMemcpyDeviceToHost, st.stream));
-    QS_CUDA(cudaMemcpyAsync(amp, oamp, sizeof(double) * 2 * K, cudaMemcpyDeviceToHost, st.stream));
-    QS_CUDA(cudaStreamSynchronize(st.stream));
+    // indices, amplitudes and the selection's state lie next to one another: one copy
+    std::vector<char> h(TL.o_ts + sizeof(TkState) - TL.o_oidx);
+    auto run = [&](TopkSelect select) {
+        topk_launch(st, K, oidx, oamp, select);
+        QS_CUDA(cudaMemcpyAsync(h.data(), oidx, h.size(), cudaMemcpyDeviceToHost, st.stream));
+        QS_CUDA(cudaStreamSynchronize(st.stream));
+        TkState ts;
+        std::memcpy(&ts, h.data() + (TL.o_ts - TL.o_oidx), sizeof(ts));
+        return ts.ok != 0;
+    };
+    // the caller waits anyway: a selection is launched only if the one before was not complete
+    int sb;
+    unsigned long long rank;
+    const bool sample = tk_sample_plan((st.dtype == QS_C128 ? 16ull : 8ull) << st.n, 1ull << st.n, K, sb, rank);
+    if (!(sample && run(TopkSelect::sampled)) && !run(TopkSelect::three_reads)) run(TopkSelect::exact);
+    std::memcpy(idx, h.data(), sizeof(uint64_t) * K);
+    std::memcpy(amp, h.data() + (TL.o_oamp - TL.o_oidx), sizeof(double) * 2 * K);
 }
 
 // ---------------------------------------------------------------------------------
