@@ -13,10 +13,21 @@ struct ChunkArgs {
     int32_t lhigh[24];  // global positions of the other local bits, ascending
     int32_t n_ops;
     uint64_t n_tiles;   // 2^(n-m)
+    // inl = 1: the pass's ops and reals come with the launch (ChunkProgram)
+    int32_t inl;
     // staged = 1: the pass's ops and reals are copied once per CTA into dynamic shared
-    // memory after the tile, at byte offsets ops_off and reals_off
+    // memory after the tile, at byte offsets ops_off and reals_off (prog_words: in 16 bytes)
     int32_t staged;
-    uint32_t ops_off, reals_off, n_reals;
+    uint32_t ops_off, reals_off, prog_words;
+};
+
+// A pass's program (ops, then reals) as a launch parameter, where it fits: a launch with 16 KB
+// of parameters follows the one before it after 3.1 us, a copy and a launch after 9.6 us, two
+// copies and a launch after 10.3 us (measured back to back), and passes over a small state take
+// little longer than that themselves.
+struct ChunkProgram {
+    static constexpr size_t kBytes = 16000;
+    alignas(16) unsigned char bytes[kBytes];
 };
 
 // One pass over the state: tiles over the local bit set `lmask`, applying `kops`

@@ -11,6 +11,7 @@
 // and the tile is written back once by TMA bulk stores.  One full HBM read + write per
 // pass, however many ops it holds.
 #include <algorithm>
+#include <cstring>
 #include <type_traits>
 
 #include "chunk.h"
@@ -115,8 +116,8 @@ __device__ void fold_hi_terms(const KOp &op, const T *src, T *dst, uint64_t base
 // (QS_PREC_IX64).  LAYERS: complex64 register phases in layers (pack_register_phases).
 template <typename T, bool DF, bool IX, bool LAYERS>
 __global__ void __launch_bounds__(kChunkThreads, 2)
-k_chunk(typename C2T<T>::type *__restrict__ psi, const ChunkArgs a, const KOp *__restrict__ ops,
-        const T *__restrict__ mats, int *__restrict__ err) {
+k_chunk(typename C2T<T>::type *__restrict__ psi, const ChunkArgs a, const unsigned char *__restrict__ program,
+        int *__restrict__ err, const __grid_constant__ ChunkProgram inline_program) {
     using V = typename C2T<T>::type;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     V *tile = (V *)smem_raw;
@@ -134,17 +135,17 @@ k_chunk(typename C2T<T>::type *__restrict__ psi, const ChunkArgs a, const KOp *_
         ptx::fence_mbar_init();
         abort_flag = 0;
     }
+    const unsigned char *const prog = a.inl ? inline_program.bytes : program;
+    const KOp *const ops = (const KOp *)prog;
+    const T *const mats = (const T *)(prog + (size_t)a.n_ops * sizeof(KOp));
     // staged: the whole pass program is copied once per CTA (tiles then need one barrier
     // per op instead of three, and no global reads of ops)
     const KOp *st_ops = (const KOp *)(smem_raw + a.ops_off);
     const T *st_m = (const T *)(smem_raw + a.reals_off);
-    if (a.staged) {
-        const uint32_t *src = (const uint32_t *)ops;
-        uint32_t *dst = (uint32_t *)(smem_raw + a.ops_off);
-        const uint32_t nw = (uint32_t)a.n_ops * (uint32_t)(sizeof(KOp) / 4);
-        for (uint32_t j = threadIdx.x; j < nw; j += blockDim.x) dst[j] = src[j];
-        T *dm = (T *)(smem_raw + a.reals_off);
-        for (uint32_t j = threadIdx.x; j < a.n_reals; j += blockDim.x) dm[j] = mats[j];
+    if (a.staged) {  // ops and reals lie behind one another here as there
+        const uint4 *src = (const uint4 *)prog;
+        uint4 *dst = (uint4 *)(smem_raw + a.ops_off);
+        for (uint32_t j = threadIdx.x; j < a.prog_words; j += blockDim.x) dst[j] = src[j];
     }
     // where run r of a tile starts, the same for every tile (a pass with more runs computes it)
     auto run_offset = [&](uint32_t r) {
@@ -235,31 +236,39 @@ template <typename T, bool DF, bool IX, bool LAYERS = false> size_t staged_limit
 
 template <typename T, bool DF, bool IX, bool LAYERS = false>
 void launch_t(DeviceState &st, const ChunkArgs &a, const std::vector<KOp> &kops, const std::vector<double> &mats) {
-    const KOp *d_ops = (const KOp *)upload_params(st, kops.data(), kops.size() * sizeof(KOp));
-    const T *d_m;
+    const size_t ops_bytes = kops.size() * sizeof(KOp);
+    const size_t reals_bytes = (DF ? 2 * sizeof(float) : sizeof(T)) * mats.size();
+    // ops, then reals in the kernel's form, in the launch parameters or in one copy
+    static thread_local ChunkProgram inl;
+    std::vector<unsigned char> big;
+    unsigned char *prog = inl.bytes;
+    const bool fits = ops_bytes + reals_bytes <= ChunkProgram::kBytes;
+    if (!fits) {
+        big.resize((ops_bytes + reals_bytes + 15) / 16 * 16);
+        prog = big.data();
+    }
+    if (ops_bytes) std::memcpy(prog, kops.data(), ops_bytes);
     if constexpr (DF) {
         // every real as a (hi, lo) float pair, same indices as the FP64 table
-        std::vector<float> pm(2 * std::max<size_t>(mats.size(), 1));
+        float *pm = (float *)(prog + ops_bytes);
         for (size_t i = 0; i < mats.size(); i++) {
             pm[2 * i] = (float)mats[i];
             pm[2 * i + 1] = (float)(mats[i] - (double)pm[2 * i]);
         }
-        d_m = (const T *)upload_params(st, pm.data(), pm.size() * sizeof(float));
     } else {
-        std::vector<T> tm(std::max<size_t>(mats.size(), 2));
+        T *tm = (T *)(prog + ops_bytes);
         for (size_t i = 0; i < mats.size(); i++) tm[i] = (T)mats[i];
-        d_m = (const T *)upload_params(st, tm.data(), tm.size() * sizeof(T));
     }
+    const unsigned char *d_prog = fits ? nullptr : (const unsigned char *)upload_params(st, big.data(), big.size());
     using V = typename C2T<T>::type;
     // stage the pass program after the tile when two CTAs per SM still fit
     ChunkArgs ca = a;
+    ca.inl = fits ? 1 : 0;
     const size_t tile_bytes = sizeof(V) << a.m;
-    const size_t ops_bytes = kops.size() * sizeof(KOp);
-    const size_t reals_bytes = (DF ? 2 * sizeof(float) : sizeof(T)) * mats.size();
     size_t smem = tile_bytes;
     ca.ops_off = (uint32_t)tile_bytes;
     ca.reals_off = (uint32_t)(tile_bytes + ops_bytes);
-    ca.n_reals = (uint32_t)mats.size();
+    ca.prog_words = (uint32_t)((ops_bytes + reals_bytes + 15) / 16);
     ca.staged = tile_bytes + ops_bytes + reals_bytes <= staged_limit<T, DF, IX, LAYERS>() ? 1 : 0;
     if (ca.staged) smem = (tile_bytes + ops_bytes + reals_bytes + 15) / 16 * 16;
     auto kern = k_chunk<T, DF, IX, LAYERS>;
@@ -272,7 +281,7 @@ void launch_t(DeviceState &st, const ChunkArgs &a, const std::vector<KOp> &kops,
         attr_set = true;
     }
     const int grid = persistent_grid((const void *)kern, kChunkThreads, smem, a.n_tiles);
-    kern<<<grid, kChunkThreads, smem, st.stream>>>((V *)st.psi, ca, d_ops, d_m, st.dev_err);
+    kern<<<grid, kChunkThreads, smem, st.stream>>>((V *)st.psi, ca, d_prog, st.dev_err, inl);
     QS_CUDA(cudaGetLastError());
     count_launch();
 }

@@ -9,7 +9,9 @@
 // two bits are both set, scalar for pairs on uniform bits and in 12 bit planes (a ripple
 // counter over the 16 registers at once) for pairs that touch register bits.
 #include <algorithm>
+#include <cstring>
 
+#include "chunk.h"
 #include "ixmath.cuh"
 #include "kops.cuh"
 #include "phasefn.h"
@@ -35,7 +37,7 @@ struct PfArgs {
     int32_t ngroups;
     int32_t table_size;
     int32_t total_pairs;
-    int32_t pad;
+    int32_t prog_words;  // table and pairs, in 16 bytes
     uint64_t n_units;
     PfGroupDev g[kPfMaxGroups];
 };
@@ -71,14 +73,14 @@ __device__ __forceinline__ double2 pf_cmul_ix(double2 a, double2 f) {
 
 template <typename T, bool IX>
 __global__ void __launch_bounds__(kPfThreads)
-k_phasefn(typename C2T<T>::type *__restrict__ psi, const PfArgs a, const uint32_t *__restrict__ pairs,
-          const typename C2T<T>::type *__restrict__ table) {
+k_phasefn(typename C2T<T>::type *__restrict__ psi, const PfArgs a, const unsigned char *__restrict__ program,
+          const __grid_constant__ ChunkProgram inline_program) {
     using V = typename C2T<T>::type;
     extern __shared__ __align__(16) unsigned char smem[];
     V *s_tab = (V *)smem;
     uint32_t *s_pairs = (uint32_t *)(s_tab + a.table_size);
-    for (int i = threadIdx.x; i < a.table_size; i += blockDim.x) s_tab[i] = table[i];
-    for (int i = threadIdx.x; i < a.total_pairs; i += blockDim.x) s_pairs[i] = pairs[i];
+    const uint4 *src = (const uint4 *)(program ? program : inline_program.bytes);  // table, then pairs
+    for (int i = threadIdx.x; i < a.prog_words; i += blockDim.x) ((uint4 *)smem)[i] = src[i];
     __syncthreads();
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const uint64_t wstep = (uint64_t)gridDim.x * (kPfThreads / 32);
@@ -158,15 +160,21 @@ void launch_t(DeviceState &st, const PhaseFn &pf) {
     }
     if ((int)pl.size() > kPfMaxPairs) fail(QS_ERR_UNSUPPORTED, "phase function with too many qubit pairs");
     a.total_pairs = (int32_t)pl.size();
-    if (pl.empty()) pl.push_back(0);
-    std::vector<V> tab(pf.table.size());
-    for (size_t i = 0; i < tab.size(); i++) {
+    // table, then pairs: in the launch parameters where they fit, else in one copy
+    const size_t table_bytes = pf.table.size() * sizeof(V), bytes = table_bytes + pl.size() * sizeof(uint32_t);
+    const size_t smem = (bytes + 15) / 16 * 16;
+    a.prog_words = (int32_t)(smem / 16);
+    static thread_local ChunkProgram inl;
+    const bool fits = smem <= ChunkProgram::kBytes;
+    std::vector<unsigned char> big(fits ? 0 : smem);
+    unsigned char *prog = fits ? inl.bytes : big.data();
+    V *tab = (V *)prog;
+    for (size_t i = 0; i < pf.table.size(); i++) {
         tab[i].x = (T)pf.table[i].real();
         tab[i].y = (T)pf.table[i].imag();
     }
-    const V *d_tab = (const V *)upload_params(st, tab.data(), tab.size() * sizeof(V));
-    const uint32_t *d_pairs = (const uint32_t *)upload_params(st, pl.data(), pl.size() * sizeof(uint32_t));
-    const size_t smem = tab.size() * sizeof(V) + (size_t)a.total_pairs * sizeof(uint32_t);
+    if (!pl.empty()) std::memcpy(prog + table_bytes, pl.data(), pl.size() * sizeof(uint32_t));
+    const unsigned char *d_prog = fits ? nullptr : (const unsigned char *)upload_params(st, big.data(), smem);
     auto kern = k_phasefn<T, IX>;
     static bool attr = false;
     if (!attr) {
@@ -175,7 +183,7 @@ void launch_t(DeviceState &st, const PhaseFn &pf) {
     }
     const uint64_t blocks = (a.n_units + kPfThreads / 32 - 1) / (kPfThreads / 32);
     const int grid = persistent_grid((const void *)kern, kPfThreads, smem, blocks);
-    kern<<<grid, kPfThreads, smem, st.stream>>>((V *)st.psi, a, d_pairs, d_tab);
+    kern<<<grid, kPfThreads, smem, st.stream>>>((V *)st.psi, a, d_prog, inl);
     QS_CUDA(cudaGetLastError());
     count_launch();
 }
