@@ -164,14 +164,18 @@ IX_HD double dot(const Num *x, const int (&idx)[K], const Num *c) {
         ep[k] = x[idx[k]].e + c[k].e;
         E = ep[k] > E ? ep[k] : E;
     }
-    int64_t acc = 0;
+    // -t is ~t + 1: the ones of all negative terms are counted and added once
+    uint64_t sum = 0;
+    uint32_t negative = 0;
 #pragma unroll
     for (int k = 0; k < K; k++) {
         const Num &a = x[idx[k]];
         const uint64_t t = shr(mulhi(a, c[k]), (uint32_t)(E - ep[k]) + HEAD);
-        const uint64_t sm = (uint64_t)(int64_t)(int32_t)(a.s ^ c[k].s);
-        acc += (int64_t)((t ^ sm) - sm);
+        const uint32_t sm = a.s ^ c[k].s;
+        sum += t ^ ((uint64_t)sm << 32 | sm);
+        negative -= sm;
     }
+    const int64_t acc = (int64_t)(sum + negative);
     const int32_t k2 = E + HEAD - 2108;
     return CVT ? encode_cvt(acc, k2) : encode_int(acc, k2);
 }

@@ -84,9 +84,11 @@ template <typename T, int NT> struct SDiag {
 
 // ---- complex128 integer-product forms (ixmath.cuh) of one-qubit dense and diagonal ops ----
 // Each thread decodes the op's constants from the matrix reals in shared memory once; every
-// fourth of its groups (iterations 0, 4, 8, ...) runs the native FP64 form, so the FP64 pipe
-// and the integer pipes share the work, as in the streaming kernel.
-constexpr uint32_t kIxNativeEvery = 4;
+// eighth of its groups (iterations 0, 8, ...) runs the native FP64 form, so the FP64 pipe and the
+// integer pipes share the work, as in the streaming kernel (a fourth there: a group's first loads
+// come from HBM; here every fourth took 128.6 ms of a 27-qubit fully connected QAOA, every eighth
+// 124.0).
+constexpr uint32_t kIxNativeEvery = 8;
 
 __device__ __forceinline__ void ix_load(const double2 &a, ix::Num (&x)[2]) {
     x[0] = ix::decode(a.x);
