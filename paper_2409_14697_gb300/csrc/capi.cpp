@@ -398,7 +398,7 @@ int qs_plan(int n_qubits, qs_dtype dt, const qs_gate *gates, size_t n_gates, con
     d.drift = RoundingDrift{};
     std::vector<Op> merged;
     std::vector<std::pair<size_t, size_t>> origin;
-    const std::vector<Pass> plan = choose_plan(ops, n_qubits, plan_params(d, o), o, merged, origin);
+    const std::vector<Pass> plan = choose_plan(ops, n_qubits, plan_params(d, o, ops), o, merged, origin);
     for (size_t p = 0; p < plan.size(); p++) {
         pass_lmask[p] = plan[p].stream ? 0 : plan[p].lmask;
         for (int i : plan[p].ops) {

@@ -130,6 +130,23 @@ PlanParams plan_params(const DeviceState &st, const qs_options &o) {
     return p;
 }
 
+PlanParams plan_params(const DeviceState &st, const qs_options &o, const std::vector<Op> &ops) {
+    PlanParams p = plan_params(st, o);
+    if (st.dtype != QS_C128 || o.chunk_m > 0 || st.n < 13 || st.n > 19) return p;
+    // 13 to 19 qubits: passes are bound by the arithmetic of the SMs that hold tiles, and 64 tiles
+    // leave more than half of them idle.  A deep circuit (6 matrices per qubit and more) gets about
+    // 256 tiles, whose extra passes stay in L2; a shallow one, whose passes take little longer
+    // than their launches, as few passes as before.  No tile below 2^8, whose ops wait on
+    // latency alone.  20-layer brickwork with 64 tiles and now: 16 qubits 822 and 488 us, 17
+    // qubits 1486 and 898, 18 qubits 2626 and 1343, 19 qubits 2783 and 2233; 16-qubit QAOA of 3
+    // layers on the complete graph 159 us with 64 tiles, 188 with 256.
+    int matrices = 0;
+    for (const Op &op : ops) matrices += !op_is_diagonal(op);
+    const int m = std::min(std::max(8, matrices >= 6 * st.n ? st.n - 8 : st.n - 6), 11);
+    if (m < st.n) p.m = m;
+    return p;
+}
+
 namespace {
 
 // One greedy pass from the first open op, local qubits restricted to low | allowed.
@@ -328,7 +345,7 @@ std::vector<Op> pass_program(const DeviceState &st, const PlanParams &pp, const 
 
 void run_planned(DeviceState &st, const std::vector<Op> &ops, const qs_options &o, qs_stats &stats) {
     const int n = st.n;
-    const PlanParams pp = plan_params(st, o);
+    const PlanParams pp = plan_params(st, o, ops);
     const double B = st.dtype == QS_C128 ? 16.0 : 8.0;
     // tiny states (no 128-byte runs): plain gate by gate
     if (n < pp.c + 1 || (B * (double)(1ull << pp.c)) < 128.0) {

@@ -23,6 +23,8 @@ struct Pass {
 };
 
 PlanParams plan_params(const DeviceState &st, const qs_options &o);
+// The same for a given circuit: the tiles of small complex128 states by its depth.
+PlanParams plan_params(const DeviceState &st, const qs_options &o, const std::vector<Op> &ops);
 // Greedy dependency-respecting partition of ops into passes.
 std::vector<Pass> make_plan(const std::vector<Op> &ops, int n, const PlanParams &pp);
 // The plan QS_MODE_AUTO / CHUNK runs: the greedy plan of ops, or, if it needs fewer passes,

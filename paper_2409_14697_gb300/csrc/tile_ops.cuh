@@ -826,7 +826,9 @@ __device__ __forceinline__ void apply_op_smem(typename C2T<T>::type *tile, const
         // with constant factors.  Diagonal blocks read from tables (F_DIAGK, F_CDIAGK,
         // F_HCDIAGK) stay native: decoding a factor per amplitude measured slower there.
         double2 *t2 = (double2 *)tile;
-        switch (op.fkind) {
+        // a thread's first group is native: with no second one there is nothing to decode for
+        const bool native = (1u << (m - op.nf)) <= blockDim.x;
+        if (!native) switch (op.fkind) {
         case F_DENSE1:
             if (op.k == D1_REAL) ix_dense1_tile<D1_REAL>(t2, op, m, sm);
             else if (op.k == D1_RX) ix_dense1_tile<D1_RX>(t2, op, m, sm);
