@@ -106,9 +106,10 @@ int qs_batch_amplitudes(qs_batch *p, uint64_t i, uint64_t off, uint64_t cnt, voi
     const uint64_t N = 1ull << b.nq[i];
     if (off > N || cnt > N - off) fail(QS_ERR_INVALID, "amplitude range out of bounds");
     const size_t B = b.dtype == QS_C128 ? 16 : 8;
+    // on the batch's stream: one wait for the run and the copy
+    QS_CUDA(cudaMemcpyAsync(host_dst, (const char *)b.d_states + (b.state_off[i] + off) * B, cnt * B,
+                            cudaMemcpyDeviceToHost, b.stream));
     QS_CUDA(cudaStreamSynchronize(b.stream));
-    QS_CUDA(cudaMemcpy(host_dst, (const char *)b.d_states + (b.state_off[i] + off) * B, cnt * B,
-                       cudaMemcpyDeviceToHost));
     QS_API_END
 }
 

@@ -280,8 +280,10 @@ void batch_build(Batch &b, const std::vector<std::vector<Op>> &circ_ops, const s
             std::vector<KOp> ko;
             std::vector<double> mt;
             const int m = __builtin_popcountll(L);
-            if (!c128 && d.reg_phases && rphase_applicable(m, kTileThreadBits)) {
-                ko = build_register_phases(fused, pos, m, kTileThreadBits, mt);
+            const int threads = rphase_threads(n, m);
+            if (!c128 && d.reg_phases && threads) {
+                ko = build_register_phases(fused, pos, m, threads, mt);
+                if (threads < kTileThreadBits) correct_drift(ko, mt);
             } else {
                 for (const Op &op : fused) ko.push_back(make_kop(op, pos, mt));
             }

@@ -316,6 +316,11 @@ void launch_chunk_pass(DeviceState &st, uint64_t lmask, const std::vector<KOp> &
             std::vector<double> packed;
             const std::vector<KOp> pk = pack_register_phases(kops, mats, (limit - taken) / sizeof(float), packed, &st.drift);
             launch_t<float, false, false, true>(st, a, pk, packed);
+        } else if (phases && a.m < kTileThreadBits + kRpBits) {
+            std::vector<KOp> ck = kops;
+            std::vector<double> cm = mats;
+            correct_drift(ck, cm);
+            launch_t<float, false, false>(st, a, ck, cm);
         } else {
             launch_t<float, false, false>(st, a, kops, mats);
         }

@@ -396,6 +396,11 @@ uint32_t tile_mask(const Op &op, const int *pos) {
 
 bool rphase_applicable(int m, int thread_bits) { return m - thread_bits == kRpBits; }
 
+int rphase_threads(int n, int m) {
+    if (rphase_applicable(m, kTileThreadBits)) return kTileThreadBits;
+    return n == m && m >= 10 && m < kTileThreadBits + kRpBits ? m - kRpBits : 0;
+}
+
 std::vector<KOp> build_register_phases(const std::vector<Op> &ops, const int *pos, int m, int thread_bits,
                                        std::vector<double> &mats, int *n_phases, bool layered) {
     if (!rphase_applicable(m, thread_bits)) fail(QS_ERR_INVALID, "register phases need m = thread bits + 5");

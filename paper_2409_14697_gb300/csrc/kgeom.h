@@ -25,6 +25,12 @@ std::vector<KOp> join_h_cdiag(const std::vector<KOp> &kops, const std::vector<do
 // complex64 tiles of 2^m amplitudes with 2^thread_bits threads: true if register phases
 // apply (m = thread_bits + kRpBits).
 bool rphase_applicable(int m, int thread_bits);
+// Thread-index bits of the register phases of an n-qubit complex64 state in tiles of 2^m
+// amplitudes, 0: none.  All threads on tiles of 2^13; 32 to 128 of them where the whole state is
+// one tile of 2^10 to 2^12 (a phase of 32 amplitudes per thread replaces several sweeps and
+// barriers: 128 circuits of 12 qubits and 60 layers in one batch 1173 -> 400 us, of 10 qubits
+// 543 -> 336).
+int rphase_threads(int n, int m);
 // Packs the pass's ops (logical qubits, tile position of qubit q = pos[q]) into register
 // phases (F_RPHASE KOps; their programs appended to `mats`).  Ops no phase can hold
 // (swaps, wider dense or diagonal blocks) become ordinary KOps in their place in the
@@ -44,6 +50,11 @@ constexpr int kPackTileBits = 9;
 // to the norm; none: tables are not corrected for it.
 std::vector<KOp> pack_register_phases(const std::vector<KOp> &kops, const std::vector<double> &mats, size_t max_reals,
                                       std::vector<double> &out, RoundingDrift *drift = nullptr);
+
+// Register phases as they are (not in layers): one member more at the end of the last, a real
+// factor that takes back what rounding the others' reals to FP32 does to the norm.  For states of
+// one tile, whose gates would otherwise run fused in FP64 and add up less of it.
+void correct_drift(std::vector<KOp> &kops, std::vector<double> &mats);
 
 // Fraction of the state's bytes one streaming application reads and writes, counting
 // whole DRAM sectors of 2^sector_bits elements.

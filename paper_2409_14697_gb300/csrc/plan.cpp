@@ -57,8 +57,9 @@ int launch_pass_ops(DeviceState &st, uint64_t lmask, const std::vector<Op> &fuse
     const int m = r;
     std::vector<KOp> kops;
     std::vector<double> mats;
-    if (!use_tc && st.dtype == QS_C64 && st.reg_phases && rphase_applicable(m, kTileThreadBits)) {
-        const std::vector<KOp> kp = build_register_phases(fused, pos, m, kTileThreadBits, mats, nullptr,
+    const int threads = rphase_threads(n, m);
+    if (!use_tc && st.dtype == QS_C64 && st.reg_phases && threads) {
+        const std::vector<KOp> kp = build_register_phases(fused, pos, m, threads, mats, nullptr,
                                                            n - m >= kPackTileBits);
         launch_chunk_pass(st, lmask, kp, mats);
         return (int)kp.size();
@@ -110,7 +111,7 @@ PlanParams plan_params(const DeviceState &st, const qs_options &o) {
     p.c = std::min(p.c, p.m);
     // the shared-memory dense path applies blocks of at most 4 qubits; complex64 register
     // phases apply gates unfused (a fused block costs more flops than its members there)
-    const bool phases = !c128 && st.reg_phases && rphase_applicable(p.m, kTileThreadBits);
+    const bool phases = !c128 && st.reg_phases && rphase_threads(st.n, p.m);
     p.fuse_k = std::min(o.fuse_k > 0 ? o.fuse_k : (phases ? 1 : 2), 4);
     // FP64 is 1/72 of FP32 on GB300: for complex128 FP64 a fused block must not add flops;
     // double-float and complex64 arithmetic run on the FP32 pipe and are cheap next to a
@@ -335,7 +336,7 @@ std::vector<Op> pass_program(const DeviceState &st, const PlanParams &pp, const 
     if (st.dtype == QS_C128) defer_hadamard_scale(pops);
     std::vector<Op> fused = fuse_ops(std::move(pops), pp.fuse_k, pp.sweep_flops, p.lmask);
     if (st.dtype == QS_C128 && st.prec == QS_PREC_FP64 && st.n - local >= 8) fused = split_one_qubit_phases(fused);
-    const bool phases = st.dtype == QS_C64 && st.reg_phases && !pp.tc && rphase_applicable(local, kTileThreadBits);
+    const bool phases = st.dtype == QS_C64 && st.reg_phases && !pp.tc && rphase_threads(st.n, local);
     if (phases && st.n - local >= kPackTileBits) fused = split_register_phases(std::move(fused));
     else if (!phases)
         fused = merge_tile_diagonals(std::move(fused), kTileDiagQubits, st.dtype == QS_C128 ? 0.5 : 4.0,

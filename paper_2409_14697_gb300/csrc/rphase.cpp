@@ -552,7 +552,65 @@ bool pack_phase(const KOp &ph, const std::vector<double> &in, size_t max_reals, 
     return true;
 }
 
+// Logarithm of the factor by which rounding a diagonal member's reals to FP32 changes the norm, its
+// entries weighted by how many amplitudes take them.
+double diagonal_drift(const double *code) {
+    const int c = (int)code[0], type = c & 7, J = (c >> 3) & 7, ea = (c >> 6) & 31, eb = (c >> 11) & 31;
+    const int len = (c >> 16) & 255;
+    const double *P = code + 1;
+    auto change = [&](int i) {  // of the squared modulus of the complex number at P[i]
+        const double r = (double)(float)P[i], m = (double)(float)P[i + 1];
+        const double e = P[i] * P[i] + P[i + 1] * P[i + 1];
+        return e > 0.0 ? (r * r + m * m - e) / e : 0.0;
+    };
+    switch (type) {
+    case RP_DIAG:
+        return ea == eb ? 0.25 * (change(0) + change(6))
+                        : 0.125 * (change(0) + change(2) + change(4) + change(6));
+    case RP_PARITY: return 0.25 * (change(0) + change(2));
+    case RP_PARITYN: {
+        const int np = (len - 2) / 3;
+        double s = 0.0, w = std::ldexp(1.0, -np);  // binomial weights
+        for (int k = 0; k <= np; k++) {
+            s += w * change(np + 2 * k);
+            w = w * (np - k) / (k + 1);
+        }
+        return 0.5 * s;
+    }
+    case RP_PH: {
+        if (J != 1) return (ea == eb ? 0.25 : 0.125) * change(0);
+        double s = 0.0;
+        for (int q = 0; q < ea; q++) s += 0.25 * change(3 * q + 1);
+        return s;
+    }
+    default: return 0.0;
+    }
+}
+
 }  // namespace
+
+void correct_drift(std::vector<KOp> &kops, std::vector<double> &mats) {
+    double drift = 0.0;
+    KOp *last = nullptr;
+    for (KOp &k : kops) {
+        if (k.fkind != F_RPHASE) continue;
+        last = &k;
+        const double *at = mats.data() + k.mat + 1;
+        for (int i = 0; i < (int)mats[(size_t)k.mat]; i++) {
+            const int code = (int)at[0], len = (code >> 16) & 255;
+            drift += rounding_drift(Matrix{at, 1 + len, 0, -1, false, false}) + diagonal_drift(at);
+            at += 1 + len;
+        }
+    }
+    // below an FP32 rounding or so there is nothing to gain; one more member has to fit
+    if (!last || std::fabs(drift) < 1e-7 || last->nmat + 3 > kMaxOpReals) return;
+    std::vector<double> prog(mats.begin() + last->mat, mats.begin() + last->mat + last->nmat);
+    prog[0] += 1.0;
+    prog.insert(prog.end(), {(double)(RP_PH | kRpAlways << 6 | kRpAlways << 11 | 2 << 16), std::exp(-drift), 0.0});
+    last->mat = (int32_t)mats.size();
+    last->nmat = (int32_t)prog.size();
+    mats.insert(mats.end(), prog.begin(), prog.end());
+}
 
 std::vector<KOp> pack_register_phases(const std::vector<KOp> &kops, const std::vector<double> &mats, size_t max_reals,
                                       std::vector<double> &out, RoundingDrift *drift) {

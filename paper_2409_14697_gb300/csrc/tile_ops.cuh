@@ -621,7 +621,7 @@ __device__ __forceinline__ void rp_store(const float2 (&v)[kRpRegs], float2 *til
     }
 }
 
-// Runs one phase: every thread of the block must call this.  Bound: the FP32 pipe and
+// Runs one phase: the 2^nt threads that hold the tile call this.  Bound: the FP32 pipe and
 // instruction issue (a brickwork pass of 26 qubits: FMA pipe 44 %, issue 56 %, HBM 18 %; the
 // rest is dependency latency at 4 warps per scheduler, the registers of 32 amplitudes).  So a
 // phase is made of few instructions: real 2x2 matrices in packed FP32 (64 per warp and gate),
@@ -911,7 +911,10 @@ __device__ __forceinline__ void apply_op_smem(typename C2T<T>::type *tile, const
         else if (op.k == 4) dense_k_smem<T, 4>(tile, op, sm, m);
         break;
     case F_RPHASE:
-        if constexpr (std::is_same<T, float>::value && RP) rphase_run<LAYERS>(tile, op, sm);
+        if constexpr (std::is_same<T, float>::value && RP) {
+            // tiles below 2^13 (never in layers): the first 2^nt threads hold them
+            if (LAYERS || !(threadIdx.x >> op.nt)) rphase_run<LAYERS>(tile, op, sm);
+        }
         break;
     default:
         break;
