@@ -41,9 +41,9 @@ std::vector<KOp> build_register_phases(const std::vector<Op> &ops, const int *po
 // Passes of 2^kPackTileBits tiles or more run their register phases in layers, with one-qubit
 // gates split into rotations and phases; smaller states wait for the host, which takes about
 // 60 us longer per pass to build them (20-layer brickwork, 21 qubits: 0.76 ms against 0.60; 22
-// qubits: 0.81 against 0.96).
+// qubits: 0.80 against 0.96).
 constexpr int kPackTileBits = 9;
-// A pass's register phases in layers: layers of a factor table and real matrices (rphase.cpp).
+// A pass's register phases in layers: layers of a factor table and shears (rphase.cpp).
 // Returns the ops with their reals re-laid in `out` (other ops unchanged), which stays within
 // max_reals, if it can, by giving later phases one layer of their members as they are; every
 // phase starts at a multiple of 4 reals.  drift: the call's account of what rounding to FP32 did

@@ -75,11 +75,12 @@ enum RpType : int {
 };
 // Phases in layers (pack_register_phases): the number of layers and three unused reals,
 // then the layers, then the tables.  A layer is
-//   h0 = real slots | class bits b << 10 | table << 13,
+//   h0 = slots of shears | slots whose bit of sigma changes after them << 5 | class bits b << 10 |
+//        table << 13,
 //   h1 = offset of its table from the program's start, h2 = the b thread-index bits that spell
 //   a thread's class c (4 bits each, bit i of c <-> i-th), h3 = members | their reals / 4 << 8,
-// then 8 reals per real slot (a real 2x2 matrix, row-major, and X M X for lanes whose bit of
-// sigma is set), then the other members (as above) up to a multiple of 4 reals; applied in this
+// then per slot of shears 4 reals (u, l and, for lanes whose bit of sigma is set, -u, -l: x += u y,
+// then y += l x on the registers with bit 0, 1 of the slot), then the other members (as above) up to a multiple of 4 reals; applied in this
 // order.  Table: register r takes the complex factor at ((r >> 1) 2^b + c) 4 + 2 (r & 1).  An
 // RP_DIAG member with slot field 1 and payload
 // (offset, lo, hi) multiplies every register by the factor at 2 c of a table, c of `a` bits named

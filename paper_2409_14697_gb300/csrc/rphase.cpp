@@ -14,9 +14,18 @@
 // Members commute unless one changes a position that the other uses, so the list is first
 // rescheduled: matrices as early as their slots' diagonals allow, diagonals gathered in as few
 // runs as the matrices between them allow.  The result is a list of layers, each a table, then
-// real 2x2 matrices on different slots, then other members as they were: the device reads one
+// shears (rotations) on different slots, then other members as they were: the device reads one
 // header per layer, where a member by itself cost about as many instructions to read as a
 // real matrix costs to apply.
+//
+// A real matrix that is a rotation, c [[1, -t], [t, 1]], is D L(k) U(-t) or L(t) U(-k) D with shears
+// L (lower) and U (upper), k = t / (1 + t^2) and D = diag(c, c (1 + t^2)).  Where the slot has a table
+// after it, or before it, D goes there and the device applies the shears.  D is by register, as the
+// shears are: a lane whose bit of sigma is set holds the rotation the other way round, which
+// negates t and k and leaves D.  |t| <= 1: a rotation by more is the one by a right angle less, a
+// sign for the table and an exchange, which only relabels the registers.  So no value grows by more
+// than sqrt(2) before its table, and an amplitude is rounded once where the matrix rounded it twice.
+// A reflection (H) is a rotation and a sign.
 //
 // The device's reals are FP32, and the rounding of an angle that a circuit repeats (Trotter
 // steps) changes the norm the same way each time.  What the matrices and the tables so far have
@@ -42,6 +51,7 @@ struct Term {
     int pos[2] = {-1, -1};
     cd d[4] = {1.0, 1.0, 1.0, 1.0};
     bool sign = false;  // only factors 1 and -1, from a sign member
+    bool fixed = false; // d by register number, not by position's bit (D of a rotation; one slot)
     int lo = 0, hi = 0, at = -1;
     uint32_t mask() const { return (np > 0 ? 1u << pos[0] : 0u) | (np > 1 ? 1u << pos[1] : 0u); }
 };
@@ -53,6 +63,8 @@ struct Matrix {
     int slot, ctl;  // ctl: operand encoding of the control, -1 if none
     bool exchange, real;
     int at = 0;
+    bool shears = false, toggle = false;  // real: as shears; then an exchange by relabelling
+    double upper = 0.0, lower = 0.0;      // x += upper y, y += lower x
 };
 
 // sigma bit of a slot as an affine function of the thread index
@@ -92,6 +104,10 @@ template <typename F> Term make_term(int ea, int eb, const F &f) {
     return t;
 }
 
+// log(1 + x) / 2 and exp(x) for the small x of roundings (|x| < 1e-5: next terms below 1e-15)
+double half_log1p(double x) { return 0.5 * x * (1.0 - 0.5 * x); }
+double exp_small(double x) { return 1.0 + x * (1.0 + 0.5 * x); }
+
 // Logarithm of the factor by which rounding the reals of a 2x2 member to FP32 changes the norm.
 double rounding_drift(const Matrix &m) {
     if (((int)m.code[0] & 7) != RP_M1) return 0.0;
@@ -101,7 +117,7 @@ double rounding_drift(const Matrix &m) {
         exact += v * v;
         rounded += f * f;
     }
-    return exact > 0.0 && rounded > 0.0 ? 0.5 * std::log1p((rounded - exact) / exact) : 0.0;
+    return exact > 0.0 && rounded > 0.0 ? half_log1p((rounded - exact) / exact) : 0.0;
 }
 
 struct Packer {
@@ -189,6 +205,106 @@ struct Packer {
         return true;
     }
 
+    // Rotations and reflections as shears where a table takes their slot's next diagonal, or its
+    // last.  keep_norm: scaled so that the norm changes as by the matrix's reals in FP32, whichever
+    // way the shears' are rounded.
+    void make_shears(bool keep_norm) {
+        const std::vector<std::pair<bool, int>> list = std::move(order);
+        order.clear();
+        order.reserve(3 * list.size());
+        terms.reserve(terms.size() + 2 * mats.size());
+        bool diagonal[kRpBits] = {false};  // on the slot until its next matrix, seen from the end
+        bool plain[kRpBits] = {false};     // an RP_R0 is still to come: no exchanges on the slot
+        std::vector<char> after(list.size(), 0), keep(list.size(), 0);
+        auto pass = [&](const Term &t) {
+            for (int k = 0; k < t.np; k++)
+                if (!t.sign && t.pos[k] >= kThreadBits) diagonal[t.pos[k] - kThreadBits] = true;
+        };
+        for (size_t i = list.size(); i-- > 0;) {
+            if (!list[i].first) {
+                pass(terms[list[i].second]);
+                continue;
+            }
+            const Matrix &m = mats[list[i].second];
+            const int code = (int)m.code[0];
+            after[i] = diagonal[m.slot];
+            keep[i] = plain[m.slot];
+            diagonal[m.slot] = false;
+            if ((code & 7) == RP_M1 && ((code >> 11) & 31) == RP_R0) plain[m.slot] = true;
+        }
+        std::fill(diagonal, diagonal + kRpBits, false);
+        for (size_t i = 0; i < list.size(); i++) {
+            if (!list[i].first) {
+                pass(terms[list[i].second]);
+                order.push_back(list[i]);
+                continue;
+            }
+            Matrix &m = mats[list[i].second];
+            const bool before = diagonal[m.slot];
+            diagonal[m.slot] = false;
+            Term d, z;
+            if ((after[i] || before) && shears(m, after[i], !keep[i], keep_norm, d, z)) {
+                auto diagonals = [&]() {
+                    add(d);
+                    if (z.d[0] != cd(1.0) || z.d[1] != cd(1.0)) add(z);
+                };
+                if (!after[i]) diagonals();
+                order.push_back(list[i]);
+                if (after[i]) diagonals();
+            } else {
+                order.push_back(list[i]);
+            }
+        }
+    }
+
+    // m as shears with the diagonal d by register and signs z, both after it or both before it.
+    static bool shears(Matrix &m, bool after, bool may_toggle, bool keep_norm, Term &d, Term &z) {
+        if (!m.real) return false;
+        const double *u = m.code + 1;
+        const bool reflection = std::fabs(u[0] + u[3]) <= 1e-15 && std::fabs(u[1] - u[2]) <= 1e-15;
+        if (!reflection && (std::fabs(u[0] - u[3]) > 1e-15 || std::fabs(u[1] + u[2]) > 1e-15)) return false;
+        double a = u[0], b = reflection ? -u[2] : u[2];  // [[a, -b], [b, a]], then a sign if a reflection
+        const bool toggle = std::fabs(a) < std::fabs(b);
+        if (toggle) {  // X Z after [[b, a], [-a, b]]
+            std::swap(a, b);
+            b = -b;
+        }
+        if (a == 0.0 || (toggle && !may_toggle)) return false;
+        m.shears = true;
+        m.toggle = toggle;
+        const double t = b / a, g = 1.0 + t * t, k = t / g;
+        double s = a;
+        if (keep_norm) {
+            // squared norm of diag(1, g) L U, rows (1, -t) and (g k, g (1 - k t)), from rounded reals
+            // (of U L diag(1, g), the other order, the same with rows and columns exchanged)
+            const double tf = (double)(float)t, kf = (double)(float)k, x = 1.0 - kf * tf;
+            const double change = (tf * tf - t * t + g * g * (kf * kf - k * k) + (g * x - 1.0) * (g * x + 1.0)) / (2.0 * g);
+            s *= exp_small(rounding_drift(m) - half_log1p(change));
+        }
+        d.np = z.np = 1;
+        d.pos[0] = z.pos[0] = kThreadBits + m.slot;
+        d.fixed = z.sign = true;
+        d.d[0] = s;
+        d.d[1] = s * g;
+        // D L(k) U(-t) or L(t) U(-k) D
+        m.upper = after ? -t : -k;
+        m.lower = after ? k : t;
+        if (after) {
+            z.d[0] = toggle ? -1.0 : 1.0;  // Z or (as X Z X) -Z
+            z.d[1] = reflection ? -1.0 : 1.0;
+            return true;
+        }
+        // before: a sign passes the shears and negates them
+        if (toggle != reflection) {
+            m.upper = -m.upper;
+            m.lower = -m.lower;
+            z.d[1] = -1.0;
+        } else if (toggle) {
+            z.d[0] = z.d[1] = -1.0;  // Z X Z = -X
+        }
+        return true;
+    }
+
     // Times: diagonal runs at even times, matrices at odd ones.  Matrices as early as their
     // operands allow; a term may go to any even time of [lo, hi].
     void schedule() {
@@ -227,10 +343,12 @@ struct Packer {
         // fewest runs: terms by their last time, each in the latest run already placed inside its
         // interval, else in a new run at its last time
         std::vector<int> by(terms.size());
-        for (size_t i = 0; i < by.size(); i++) by[i] = (int)i;
         const int end = last ? last + 1 : 0;
         for (Term &t : terms) t.hi = std::min(t.hi, end);
-        std::stable_sort(by.begin(), by.end(), [&](int a, int b) { return terms[a].hi < terms[b].hi; });
+        std::vector<int> first((size_t)end + 2, 0);
+        for (const Term &t : terms) first[(size_t)t.hi + 1]++;
+        for (int i = 0; i <= end; i++) first[(size_t)i + 1] += first[(size_t)i];
+        for (size_t i = 0; i < terms.size(); i++) by[(size_t)first[(size_t)terms[i].hi]++] = (int)i;
         std::vector<int> runs;
         for (int i : by) {
             Term &t = terms[i];
@@ -262,76 +380,112 @@ std::pair<double, double> emit_table(const Packer &p, const Table &tb, double sc
         if ((tb.bits >> i) & 1u) bit[nb++] = i;
     const size_t at = out.size();
     out.resize(at + ((size_t)64 << nb));
-    // factors in logical order (slot bits x), real and imaginary parts
+    // A class's factors in logical order (slot bits x) are a number, a pair per slot and, for all
+    // classes, a product over pairs of slots.
     struct Factors {
         double re[kRegs], im[kRegs];
-        void mul(int x, cd z) {
-            const double r = re[x] * z.real() - im[x] * z.imag();
-            im[x] = re[x] * z.imag() + im[x] * z.real();
-            re[x] = r;
-        }
     };
-    Factors fixed;  // the part that only slots choose
-    std::fill(fixed.re, fixed.re + kRegs, scale);
-    std::fill(fixed.im, fixed.im + kRegs, 0.0);
+    cd number = scale, slot[kRpBits][2];
+    for (auto &f : slot) f[0] = f[1] = 1.0;
+    double by_register[kRegs], weight[kRegs];
+    by_register[0] = weight[0] = 1.0;
+    double fixed[kRpBits][2];
+    for (auto &f : fixed) f[0] = f[1] = 1.0;
+    Factors two;
+    bool any_two = false;
     std::vector<const Term *> mixed;
     uint32_t chooses = 0;  // thread bits in terms (the others of the class only permute)
     for (int i : tb.terms) {
         const Term &t = p.terms[i];
-        if (t.np > 0 && t.pos[0] < kThreadBits) {
+        const int a = t.np > 0 ? t.pos[0] - kThreadBits : 0;
+        if (t.fixed) {
+            for (int h = 0; h < 2; h++) fixed[a][h] *= t.d[h].real();
+        } else if (t.np == 0) {
+            number *= t.d[0];
+        } else if (a < 0) {
             mixed.push_back(&t);
             chooses |= t.mask();
-            continue;
+        } else if (t.np == 1) {
+            for (int h = 0; h < 2; h++) slot[a][h] *= t.d[h];
+        } else {
+            const int b = t.pos[1] - kThreadBits;
+            for (int x = 0; x < kRegs; x++) {
+                const cd z = t.d[((x >> a) & 1) + 2 * ((x >> b) & 1)];
+                const double re = any_two ? two.re[x] : 1.0, im = any_two ? two.im[x] : 0.0;
+                two.re[x] = re * z.real() - im * z.imag();
+                two.im[x] = re * z.imag() + im * z.real();
+            }
+            any_two = true;
         }
-        const int a = t.np > 0 ? t.pos[0] - kThreadBits : 0, b = t.np == 2 ? t.pos[1] - kThreadBits : 0;
-        for (int x = 0; x < kRegs; x++)
-            fixed.mul(x, t.d[(t.np > 0 ? (x >> a) & 1 : 0) + (t.np == 2 ? 2 * ((x >> b) & 1) : 0)]);
     }
-    Factors f = fixed;
-    double exact = 0.0, rounded = 0.0, exact_f = 0.0, rounded_f = 0.0;
-    auto weigh = [&]() {  // a class's factors, whatever their order
-        exact_f = rounded_f = 0.0;
-        for (int x = 0; x < kRegs; x++) {
-            const double r = (double)(float)f.re[x], i = (double)(float)f.im[x];
-            exact_f += f.re[x] * f.re[x] + f.im[x] * f.im[x];
-            rounded_f += r * r + i * i;
+    double inverse[kRpBits][2];  // squares
+    for (int j = 0; j < kRpBits; j++)
+        for (int h = 0; h < 2; h++) inverse[j][h] = fixed[j][h] == 1.0 ? 1.0 : 1.0 / (fixed[j][h] * fixed[j][h]);
+    for (int j = 0; j < kRpBits; j++)
+        for (int x = 0; x < (1 << j); x++) {
+            by_register[x + (1 << j)] = by_register[x] * fixed[j][1];
+            by_register[x] *= fixed[j][0];
+            weight[x + (1 << j)] = weight[x] * inverse[j][1];
+            weight[x] *= inverse[j][0];
         }
-    };
-    weigh();
+    Factors f;
+    double exact = 0.0, rounded = 0.0, exact_f = 0.0, rounded_f = 0.0;
     uint32_t made = ~0u;  // the chosen bits that f was made for
     for (int c = 0; c < (1 << nb); c++) {
         uint32_t tid = 0;
         for (int i = 0; i < nb; i++) tid |= (uint32_t)((c >> i) & 1) << bit[i];
-        if (!mixed.empty() && (tid & chooses) != made) {
+        const bool make = (tid & chooses) != made;
+        if (make) {
             made = tid & chooses;
-            f = fixed;
+            cd n = number, s[kRpBits][2];
+            std::copy(&slot[0][0], &slot[0][0] + 2 * kRpBits, &s[0][0]);
             for (const Term *t : mixed) {
                 const int x0 = (tid >> t->pos[0]) & 1;
-                if (t->np == 2 && t->pos[1] >= kThreadBits) {
-                    const int j = t->pos[1] - kThreadBits;
-                    for (int h = 0; h < 2; h++)
-                        if (t->d[x0 + 2 * h] != cd(1.0))
-                            for (int x = 0; x < kRegs; x++)
-                                if (((x >> j) & 1) == h) f.mul(x, t->d[x0 + 2 * h]);
-                } else {
-                    const cd z = t->d[x0 + (t->np == 2 ? 2 * ((tid >> t->pos[1]) & 1) : 0)];
-                    for (int x = 0; x < kRegs; x++) f.mul(x, z);
+                if (t->np == 2 && t->pos[1] >= kThreadBits)
+                    for (int h = 0; h < 2; h++) s[t->pos[1] - kThreadBits][h] *= t->d[x0 + 2 * h];
+                else n *= t->d[x0 + (t->np == 2 ? 2 * ((tid >> t->pos[1]) & 1) : 0)];
+            }
+            f.re[0] = n.real();
+            f.im[0] = n.imag();
+            for (int j = 0; j < kRpBits; j++) {
+                const double ar = s[j][0].real(), ai = s[j][0].imag(), br = s[j][1].real(), bi = s[j][1].imag();
+                for (int x = 0; x < (1 << j); x++) {
+                    const double re = f.re[x], im = f.im[x];
+                    f.re[x + (1 << j)] = re * br - im * bi;
+                    f.im[x + (1 << j)] = re * bi + im * br;
+                    f.re[x] = re * ar - im * ai;
+                    f.im[x] = re * ai + im * ar;
                 }
             }
-            weigh();
+            if (any_two)
+                for (int x = 0; x < kRegs; x++) {
+                    const double re = f.re[x];
+                    f.re[x] = re * two.re[x] - f.im[x] * two.im[x];
+                    f.im[x] = re * two.im[x] + f.im[x] * two.re[x];
+                }
         }
-        exact += exact_f;
-        rounded += rounded_f;
         int sg = 0;  // register r holds the amplitude whose slot bits are r ^ sigma
         for (int j = 0; j < kRpBits; j++)
             sg |= (int)((__builtin_popcount(p.sigma[j].bits & tid) & 1) ^ (p.sigma[j].one ? 1 : 0)) << j;
         double *o = out.data() + at + 4 * (size_t)c;
-        for (int r = 0; r < kRegs; r += 2, o += (size_t)4 << nb) {
-            o[0] = f.re[r ^ sg];
-            o[1] = f.im[r ^ sg];
-            o[2] = f.re[(r + 1) ^ sg];
-            o[3] = f.im[(r + 1) ^ sg];
+        const size_t step = (size_t)4 << nb;
+        for (int r = 0; r < kRegs; r++) {
+            double *e = o + (size_t)(r >> 1) * step + 2 * (r & 1);
+            e[0] = f.re[r ^ sg] * by_register[r];
+            e[1] = f.im[r ^ sg] * by_register[r];
         }
+        if (make) {  // for all classes of these factors, whose order differs; an amplitude counts by
+                     // what it was before a rotation's D
+            exact_f = rounded_f = 0.0;
+            for (int r = 0; r < kRegs; r++) {
+                const double *e = o + (size_t)(r >> 1) * step + 2 * (r & 1);
+                const double a = (double)(float)e[0], b = (double)(float)e[1];
+                exact_f += weight[r] * (e[0] * e[0] + e[1] * e[1]);
+                rounded_f += weight[r] * (a * a + b * b);
+            }
+        }
+        exact += exact_f;
+        rounded += rounded_f;
     }
     return {exact, rounded};
 }
@@ -359,7 +513,7 @@ struct Layer {
     int table = -1;      // index into the tables' offsets, -1: none
     int class_bits = 0;  // number of thread bits that spell a class
     uint32_t class_pos = 0;
-    const Matrix *real[kRpBits] = {nullptr};
+    const Matrix *real[kRpBits] = {nullptr};  // as shears
     int members = 0;          // other members, in order
     std::vector<double> raw;
     uint32_t raw_uses = 0;    // slots they change or read
@@ -372,6 +526,7 @@ bool pack_phase(const KOp &ph, const std::vector<double> &in, size_t max_reals, 
     Packer p(ph);
     if (ph.nt != kThreadBits || !p.decode(in.data() + ph.mat)) return false;
     if (p.terms.empty()) return false;
+    p.make_shears(drift != nullptr);
     p.schedule();
     int last = 0;
     for (const Matrix &m : p.mats) last = std::max(last, m.at);
@@ -402,11 +557,17 @@ bool pack_phase(const KOp &ph, const std::vector<double> &in, size_t max_reals, 
             const int b = t.np > 1 ? encode_position(t.pos[1]) : a;
             if (t.sign) {
                 // a sign member's term is -1 exactly where its one or two positions are 1, or
-                // nowhere (paired with a bit that is 0)
+                // nowhere (paired with a bit that is 0); a rotation's may be -1 where they are 0
                 const cd v = t.np == 0 ? t.d[0] : t.d[t.np == 2 ? 3 : 1];
+                if (t.np == 1 && t.d[0] == cd(-1.0)) {
+                    pairs.push_back((double)(kRpAlways | kRpAlways << 5));
+                    if (v == cd(1.0)) pairs.push_back((double)(a | b << 5));
+                    if (pairs.size() >= 7) flush();
+                    continue;
+                }
                 if (v != cd(-1.0)) continue;
                 pairs.push_back((double)(a | b << 5));
-                if (pairs.size() == 8) flush();
+                if (pairs.size() >= 7) flush();
             } else if (t.np < 2) {
                 const cd d0 = t.d[0], d1 = t.np ? t.d[1] : t.d[0];
                 raw(RP_PARITY, 0, a, kRpNever, {d0.real(), d0.imag(), d1.real(), d1.imag()});
@@ -422,10 +583,11 @@ bool pack_phase(const KOp &ph, const std::vector<double> &in, size_t max_reals, 
         const uint32_t slot = 1u << (kThreadBits + m.slot);
         const int c = m.ctl >= 0 ? position_of(m.ctl) : kNone;
         if (layers.empty()) layers.emplace_back();
-        if (m.real) {
+        if (m.shears) {
             if (layers.back().real[m.slot] || (layers.back().raw_uses & slot)) layers.emplace_back();
             Layer &l = layers.back();
             l.real[m.slot] = &m;
+            if (m.toggle) p.sigma[m.slot].one = !p.sigma[m.slot].one;
             return;
         }
         Layer &l = layers.back();
@@ -437,33 +599,42 @@ bool pack_phase(const KOp &ph, const std::vector<double> &in, size_t max_reals, 
         if (c == kOn) p.sigma[m.slot].one = !p.sigma[m.slot].one;
         else if (c >= 0 && c < kThreadBits) p.sigma[m.slot].bits ^= 1u << c;
     };
+    // terms (even times) and matrices (odd ones), each in circuit order
+    std::vector<int> begin((size_t)last + 2, 0), list(p.order.size());
+    auto time_of = [&](const std::pair<bool, int> &o) { return o.first ? p.mats[o.second].at : p.terms[o.second].at; };
+    for (const auto &o : p.order) begin[(size_t)time_of(o) + 1]++;
+    for (size_t i = 1; i < begin.size(); i++) begin[i] += begin[i - 1];
+    {
+        std::vector<int> next(begin);
+        for (const auto &o : p.order) list[(size_t)next[(size_t)time_of(o)]++] = o.second;
+    }
     for (int time = 0; time <= last; time++) {
+        const int *const first = list.data() + begin[(size_t)time], *const end = list.data() + begin[(size_t)time + 1];
         if (time & 1) {
-            for (const auto &o : p.order)
-                if (o.first && p.mats[o.second].at == time) matrix(p.mats[o.second]);
+            for (const int *i = first; i < end; i++) matrix(p.mats[*i]);
             continue;
         }
+        if (first == end) continue;
         std::vector<Table> tabs;
         Table uniform;  // terms that no slot chooses
         std::vector<int> alone, free_terms;
         bool signs_only = true;
-        for (const Term &t : p.terms) signs_only = signs_only && !(t.at == time && !t.sign);
-        for (size_t i = 0; i < p.terms.size(); i++) {
-            const Term &t = p.terms[i];
-            if (t.at != time) continue;
+        for (const int *i = first; i < end; i++) signs_only = signs_only && p.terms[*i].sign;
+        for (const int *i = first; i < end; i++) {
+            const Term &t = p.terms[*i];
             if (signs_only) {  // a sign costs less than a table's complex multiply
-                alone.push_back((int)i);
+                alone.push_back(*i);
                 continue;
             }
             if ((t.mask() & kSlotMask) == 0) {
-                free_terms.push_back((int)i);
+                free_terms.push_back(*i);
                 continue;
             }
             uint32_t need = t.mask() & ((1u << kThreadBits) - 1u);
             for (int k = 0; k < t.np; k++)
-                if (t.pos[k] >= kThreadBits) need |= p.sigma[t.pos[k] - kThreadBits].bits;
+                if (t.pos[k] >= kThreadBits && !t.fixed) need |= p.sigma[t.pos[k] - kThreadBits].bits;
             if (__builtin_popcount(need) > kRpMaxClassBits) {
-                alone.push_back((int)i);
+                alone.push_back(*i);
                 continue;
             }
             Table *to = nullptr;
@@ -474,7 +645,7 @@ bool pack_phase(const KOp &ph, const std::vector<double> &in, size_t max_reals, 
                 to = &tabs.back();
             }
             to->bits |= need;
-            to->terms.push_back((int)i);
+            to->terms.push_back(*i);
         }
         // factors without a register position: in a table that has room for their bits
         for (int i : free_terms) {
@@ -494,10 +665,10 @@ bool pack_phase(const KOp &ph, const std::vector<double> &in, size_t max_reals, 
             double fix = 0.0;
             if (drift && std::fabs(account.open) < kMaxDriftFix)
                 fix = std::min(std::max(account.fixed - account.open, -kMaxDriftFix), kMaxDriftFix) - account.fixed;
-            const auto sums = emit_table(p, tb, std::exp(fix), tables);
+            const auto sums = emit_table(p, tb, exp_small(fix), tables);
             account.fixed += fix;
             account.open += fix;
-            if (sums.first > 0.0) account.open += 0.5 * std::log1p((sums.second - sums.first) / sums.first);
+            if (sums.first > 0.0) account.open += half_log1p((sums.second - sums.first) / sums.first);
         }
         if (!uniform.terms.empty()) {
             double lo = 0.0, hi = 0.0;
@@ -519,7 +690,7 @@ bool pack_phase(const KOp &ph, const std::vector<double> &in, size_t max_reals, 
     for (Layer &l : layers) {
         while (l.raw.size() % 4) l.raw.push_back(0.0);
         size += 4 + l.raw.size();
-        for (const Matrix *m : l.real) size += m ? 8 : 0;
+        for (const Matrix *m : l.real) size += m ? 4 : 0;
     }
     const size_t pad = (4 - out.size() % 4) % 4;
     if (pad + size + tables.size() > max_reals || layers.size() > 1000) return false;
@@ -530,14 +701,14 @@ bool pack_phase(const KOp &ph, const std::vector<double> &in, size_t max_reals, 
     out.insert(out.end(), {(double)layers.size(), 0.0, 0.0, 0.0});
     for (Layer &l : layers) {
         uint32_t mask = 0;
-        for (int j = 0; j < kRpBits; j++) mask |= l.real[j] ? 1u << j : 0u;
+        for (int j = 0; j < kRpBits; j++)
+            if (const Matrix *m = l.real[j]) mask |= (m->toggle ? 33u : 1u) << j;
         out.push_back((double)(mask | (uint32_t)l.class_bits << 10 | (l.table >= 0 ? 1u << 13 : 0u)));
         out.push_back(l.table >= 0 ? (double)(size + table_at[(size_t)l.table]) : 0.0);
         out.push_back((double)l.class_pos);
         out.push_back((double)(l.members | (uint32_t)(l.raw.size() / 4) << 8));
         for (const Matrix *m : l.real)
-            if (m) out.insert(out.end(), {m->code[1], m->code[2], m->code[3], m->code[4],   // M
-                                          m->code[4], m->code[3], m->code[2], m->code[1]}); // X M X
+            if (m) out.insert(out.end(), {m->upper, m->lower, -m->upper, -m->lower});
         // a thread table's member names its table by number until here
         for (size_t at = 0, k = 0; k < (size_t)l.members; k++) {
             const int code = (int)l.raw[at];

@@ -481,11 +481,18 @@ __device__ __forceinline__ void rp_class_table(float2 (&v)[kRpRegs], const float
     }
 }
 
-// a layer's real matrix on slot J; X M X (the second 4 reals) in lanes whose bit of sigma is set
+// a layer's shears on slot J: x += u y, then y += l x, u and l negated in lanes whose bit of sigma is
+// set (the second 2 reals): one packed multiply-add per amplitude, in place (no copies)
 template <int J>
-__device__ __forceinline__ void rp_layer_real(float2 (&v)[kRpRegs], const float4 *P, uint32_t sigma) {
-    const float4 q = P[(sigma >> J) & 1u];
-    rp_mr<J>(v, q.x, q.y, q.z, q.w);
+__device__ __forceinline__ void rp_shears(float2 (&v)[kRpRegs], const float4 *P, uint32_t sigma) {
+    const float2 q = ((const float2 *)P)[(sigma >> J) & 1u];
+    const float2 U = make_float2(q.x, q.x), L = make_float2(q.y, q.y);
+#pragma unroll
+    for (int r = 0; r < kRpRegs; r++)
+        if (!(r & (1 << J))) v[r] = __ffma2_rn(U, v[r | (1 << J)], v[r]);
+#pragma unroll
+    for (int r = 0; r < kRpRegs; r++)
+        if (r & (1 << J)) v[r] = __ffma2_rn(L, v[r & ~(1 << J)], v[r]);
 }
 
 __device__ __forceinline__ void rp_ph(float2 (&v)[kRpRegs], float pr, float pi, uint32_t K) {
@@ -621,14 +628,16 @@ __device__ __forceinline__ void rp_store(const float2 (&v)[kRpRegs], float2 *til
     }
 }
 
-// Runs one phase: the 2^nt threads that hold the tile call this.  Bound: the FP32 pipe and
-// instruction issue (a brickwork pass of 26 qubits: FMA pipe 44 %, issue 56 %, HBM 18 %; the
-// rest is dependency latency at 4 warps per scheduler, the registers of 32 amplitudes).  So a
-// phase is made of few instructions: real 2x2 matrices in packed FP32 (64 per warp and gate),
-// one complex multiply and half a load per amplitude for all diagonals between two layers of
-// matrices, one read of the program per layer.  28-qubit brickwork of 40 layers 117.5 -> 67.0 ms
-// (74.4 ms before offsets in bytes and run offsets made once), 30-qubit QAOA p = 4 99.6 -> 71.6
-// ms, 25-qubit Trotter circuit of 16 steps 7.4 -> 5.0 ms.  LAYERS: the program is in layers
+// Runs one phase: the 2^nt threads that hold the tile call this.  Bound: instruction issue and
+// fixed latencies (a brickwork pass of 26 qubits issues in 55 % of the cycles, FMA pipe 35 %, shared
+// memory 33 %, HBM 18 %; 4 warps per scheduler, the registers of 32 amplitudes, wait 1.3 of 6
+// cycles per instruction).  So a phase is made of few instructions: a rotation is two shears in
+// place, 32 packed multiply-adds per warp (as a matrix 64; as (1, -t; t, 1) 32 and 32 moves, since
+// both results need both old values: 65.7 ms in the case below), all diagonals between two layers
+// of rotations one complex multiply and half a load per amplitude, one read of the program per
+// layer.  28-qubit brickwork of 40 layers 117.5 ms with members alone, 74.4 in layers, 66.8 with
+// offsets in bytes and run offsets made once, 56.3 with shears; 30-qubit QAOA p = 4 99.6, 71.6 and,
+// with shears, 69.4 ms; 25-qubit Trotter circuit of 16 steps 7.4, 4.94, 4.42 ms.  LAYERS: the program is in layers
 // (passes of many tiles); else it is a member count and the members.  Two instances, since
 // reading both in one cost the plain form 12 % (small states wait for single tiles).
 template <bool LAYERS>
@@ -644,7 +653,7 @@ __device__ __forceinline__ void rphase_run(float2 *tile, const KOp &ph, const fl
     // at: the next real of the program; layers and members left to do, counted in one register
     uint32_t at = LAYERS ? 4u : 1u, left = rp_int(prog[0]) << (LAYERS ? 8 : 0);
     while (left) {
-        if (LAYERS && !(left & 255u)) {  // the next layer's table and real matrices
+        if (LAYERS && !(left & 255u)) {  // the next layer's table and shears
             const float4 *P = (const float4 *)(prog + at);
             const float4 h = *P++;
             const uint32_t h0 = rp_int(h.x);
@@ -656,11 +665,12 @@ __device__ __forceinline__ void rphase_run(float2 *tile, const KOp &ph, const fl
                 else rp_class_table<0>(v, table + rp_class(rp_int(h.z), 0u, nb, tid), 1u << nb);
             }
             const float4 *const P0 = P;
-            if (h0 & 1u) { rp_layer_real<0>(v, P, sigma); P += 2; }
-            if (h0 & 2u) { rp_layer_real<1>(v, P, sigma); P += 2; }
-            if (h0 & 4u) { rp_layer_real<2>(v, P, sigma); P += 2; }
-            if (h0 & 8u) { rp_layer_real<3>(v, P, sigma); P += 2; }
-            if (h0 & 16u) { rp_layer_real<4>(v, P, sigma); P += 2; }
+            if (h0 & 1u) rp_shears<0>(v, P++, sigma);
+            if (h0 & 2u) rp_shears<1>(v, P++, sigma);
+            if (h0 & 4u) rp_shears<2>(v, P++, sigma);
+            if (h0 & 8u) rp_shears<3>(v, P++, sigma);
+            if (h0 & 16u) rp_shears<4>(v, P++, sigma);
+            sigma ^= (h0 >> 5) & 31u;
             left += (rp_int(((const float *)P0)[-1]) & 255u) - 256u;
             at = (uint32_t)((const float *)P - prog);
             continue;

@@ -13,7 +13,7 @@
 
 namespace {
 
-int g_slot_tables = 0, g_thread_tables = 0, g_packed = 0, g_kept = 0;
+int g_slot_tables = 0, g_thread_tables = 0, g_packed = 0, g_kept = 0, g_shears = 0, g_toggles = 0;
 
 // Factor tables on the tile: per thread and register, entry(r, class).
 template <typename F>
@@ -30,6 +30,26 @@ void apply_table(State &tile, const KOp &ph, const uint32_t *sig_bits, const boo
             for (int j = 0; j < kRpBits; j++)
                 if (((r ^ sigma) >> j) & 1u) x |= 1u << ph.pos[j];
             tile[x] *= entry(r, c);
+        }
+    }
+}
+
+// x += u y, y += l x on the amplitudes that registers with bit j clear and set hold; in threads whose
+// bit of sigma is set, those are the amplitudes with that position set and clear, and u, l negated.
+void apply_shears(State &tile, const KOp &ph, const uint32_t *sig_bits, const bool *sig_one, int j, double u, double l) {
+    for (uint32_t tid = 0; tid < (1u << ph.nt); tid++) {
+        const bool s = (__builtin_popcount(sig_bits[j] & tid) & 1) ^ (int)sig_one[j];
+        uint64_t base = 0;
+        for (int b = 0; b < ph.nt; b++) base |= (uint64_t)((tid >> b) & 1u) << (uint32_t)((ph.off[0] >> (4 * b)) & 15u);
+        for (uint32_t r = 0; r < 32; r++) {
+            if ((r >> j) & 1u) continue;
+            uint64_t x = base;
+            for (int i = 0; i < kRpBits; i++)
+                if ((r >> i) & 1u) x |= 1ull << ph.pos[i];
+            const uint64_t y = x | 1ull << ph.pos[j];
+            cd &a = tile[s ? y : x], &b = tile[s ? x : y];
+            a += (s ? -u : u) * b;
+            b += (s ? -l : l) * a;
         }
     }
 }
@@ -69,15 +89,24 @@ void apply_packed(State &tile, int m, const KOp &ph, const std::vector<double> &
         const double *P = at + 4;
         for (int j = 0; j < kRpBits; j++) {
             if (!((h0 >> j) & 1u)) continue;
-            check(P[4] == P[3] && P[5] == P[2] && P[6] == P[1] && P[7] == P[0], "conjugated matrix", trial);
-            double code[5] = {(double)(RP_M1 | j << 3 | RP_REAL << 11 | 4 << 16), P[0], P[1], P[2], P[3]};
-            member(code, 5);
-            P += 8;
+            check(P[2] == -P[0] && P[3] == -P[1] && std::fabs(P[0]) <= 1.0 && std::fabs(P[1]) <= 1.0, "shears", trial);
+            apply_shears(tile, ph, sig_bits, sig_one, j, P[0], P[1]);
+            g_shears++;
+            P += 4;
         }
+        for (int j = 0; j < kRpBits; j++)
+            if ((h0 >> (5 + j)) & 1u) {  // an exchange that relabels
+                for (uint64_t x = 0; x < tile.size(); x++)
+                    if ((x >> ph.pos[j]) & 1u) std::swap(tile[x], tile[x ^ (1ull << ph.pos[j])]);
+                sig_one[j] = !sig_one[j];
+                g_toggles++;
+            }
         const double *mm = P;
         for (int i = 0; i < (int)(h3 & 255u); i++) {
             const int code = (int)mm[0], type = code & 7, J = (code >> 3) & 7, ea = (code >> 6) & 31;
             const int len = (code >> 16) & 255;
+            if (type == RP_M1 && ((code >> 11) & 31) == RP_R0)
+                check(sig_bits[J] == 0 && !sig_one[J], "RP_R0 on a slot that sigma relabels", trial);
             if (type == RP_DIAG && J != 0) {
                 g_thread_tables++;
                 const size_t off = (size_t)mm[1];
@@ -172,6 +201,25 @@ int main(int argc, char **argv) {
                     for (int b = a + 1; b < n; b++) dense.push_back(gate(s & 1 ? QS_CP : QS_RZZ, {a, b}, ang(g)));
                 for (int q = 0; q < n; q++) dense.push_back(gate(QS_H, {q}));
             }
+            // rotations and reflections by any angle, at the ends of the shears' range too, with their
+            // diagonals before or after them
+            for (bool first : {false, true}) {
+                std::vector<Op> turns;
+                const double edge[6] = {0.0, M_PI / 4, M_PI / 2, M_PI, 1e-9, -M_PI / 4};
+                for (int q = 0; q < n; q++) {
+                    const double a = (q + trial) % 3 ? ang(g) : edge[(q + trial) / 3 % 6], c = std::cos(a), s = std::sin(a);
+                    Op t;
+                    t.kind = K_DENSE1;
+                    t.k = 1;
+                    t.q[0] = q;
+                    if (q & 1) t.m = {cd(c), cd(s), cd(s), cd(-c)};
+                    else t.m = {cd(c), cd(-s), cd(s), cd(c)};
+                    if (first) turns.push_back(t);
+                    turns.push_back(gate(QS_P, {q}, ang(g)));
+                    if (!first) turns.push_back(t);
+                }
+                check_pack(g, turns, 10000, trial, true);
+            }
             for (const auto *ops : {&chain, &phases, &dense})
                 for (size_t limit : {(size_t)10000, (size_t)2500, (size_t)0}) {
                     check_pack(g, *ops, limit, trial, true);
@@ -182,7 +230,7 @@ int main(int argc, char **argv) {
             g_bad++;
         }
     }
-    check(g_slot_tables > 0 && g_thread_tables > 0 && g_packed > 0 && g_kept > 0, "packing not exercised", -1);
+    check(g_slot_tables > 0 && g_thread_tables > 0 && g_shears > 0 && g_toggles > 0 && g_packed > 0 && g_kept > 0, "packing not exercised", -1);
     std::printf("%s (%d slot tables, %d thread tables, %d phases packed, %d kept)\n", g_bad ? "FAIL" : "OK",
                 g_slot_tables, g_thread_tables, g_packed, g_kept);
     return g_bad ? 1 : 0;

@@ -338,3 +338,29 @@ def test_register_phases_in_layers(qs, n):
     got, _ = _run_c64(qs, n, psi0, gates)
     assert np.max(np.abs(got - want)) <= TOL_C64
     assert fidelity_gap(got, want) <= 1e-6
+
+
+@pytest.mark.parametrize("n", [22, 23])
+def test_rotations_as_shears(qs, n):
+    """Layered register phases turn rotations and reflections into shears, exchanges by relabelling
+    and factors of a table: RY and U3 at the ends of the shears' range (0, a right angle and either
+    side of it) and in between, H, with phases before or after them, exchanges and gates that follow
+    on relabelled slots, against the oracle.  The bound is that of the other phases: the shears round
+    once per amplitude where the matrix rounded twice."""
+    r = np.random.default_rng(n)
+    edge = [0.0, np.pi / 2, np.pi, -np.pi / 2, 1.5 * np.pi, 1e-6, np.pi / 2 + 1e-6, np.pi / 2 - 1e-6]
+    gates = []
+    for layer in range(6):
+        for q in range(n):
+            a = float(edge[(q + layer) % 8] if (q + layer) % 2 else r.uniform(-6.28, 6.28))
+            phase = ("p", (q,), (float(r.uniform(0, 6.28)),))
+            turn = [("ry", (q,), (a,)), ("h", (q,), ()), ("u3", (q,), (a, 0.3, 1.1))][(q + layer) % 3]
+            gates += [turn, phase] if layer % 2 else [phase, turn]
+        for a in range(layer % 2, n - 1, 2):
+            gates.append((("cnot", "cz", "cnot")[layer % 3], (a, a + 1), ()))
+        gates += [("x", (layer,), ()), ("ry", (layer,), (0.7,)), ("u3", (layer,), (2.2, 0.4, 0.5))]
+    psi0 = inputs.gaussian_state(n, seed=n).astype(np.complex64)
+    want = oracle.run(psi0.astype(np.complex128), n, gates)
+    got, _ = _run_c64(qs, n, psi0, gates)
+    assert np.max(np.abs(got - want)) <= TOL_C64
+    assert fidelity_gap(got, want) <= 1e-6
