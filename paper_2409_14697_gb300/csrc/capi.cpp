@@ -154,7 +154,7 @@ void run_circuit(DeviceState &d, const std::vector<Op> &ops, const qs_options &o
         fail(QS_ERR_INVALID, "unknown precision mode");
     d.prec = o.precision == QS_PREC_DF32 ? QS_PREC_DF32 : QS_PREC_FP64;
     d.ix = o.precision == QS_PREC_IX64 || o.precision == QS_PREC_DEFAULT;
-    d.reg_phases = (o.flags & QS_OPT_NO_REG_PHASES) == 0;
+    d.reg_phases = use_register_phases(ops, d.n, o);
     d.drift = RoundingDrift{};
     const uint64_t l0 = g_launches.load();
     arena_begin(d);
@@ -394,7 +394,7 @@ int qs_plan(int n_qubits, qs_dtype dt, const qs_gate *gates, size_t n_gates, con
     DeviceState d;
     d.n = n_qubits;
     d.dtype = dt;
-    d.reg_phases = (o.flags & QS_OPT_NO_REG_PHASES) == 0;
+    d.reg_phases = use_register_phases(ops, n_qubits, o);
     d.drift = RoundingDrift{};
     std::vector<Op> merged;
     std::vector<std::pair<size_t, size_t>> origin;

@@ -308,11 +308,14 @@ void launch_chunk_pass(DeviceState &st, uint64_t lmask, const std::vector<KOp> &
         else if (st.ix) launch_t<double, false, true>(st, a, kops, mats);
         else launch_t<double, false, false>(st, a, kops, mats);
     } else {
-        bool phases = false;
-        for (const KOp &k : kops) phases |= k.fkind == F_RPHASE;
+        bool phases = false, layers = false;
+        for (const KOp &k : kops) {
+            phases |= k.fkind == F_RPHASE;
+            layers |= k.fkind == F_RPHASE && k.nf;
+        }
         const size_t taken = (B << a.m) + kops.size() * sizeof(KOp);
         const size_t limit = staged_limit<float, false, false, true>();
-        if (phases && n - a.m >= kPackTileBits && taken < limit) {
+        if (layers && n - a.m >= kPackTileBits && taken < limit) {
             std::vector<double> packed;
             const std::vector<KOp> pk = pack_register_phases(kops, mats, (limit - taken) / sizeof(float), packed, &st.drift);
             launch_t<float, false, false, true>(st, a, pk, packed);

@@ -485,6 +485,7 @@ std::vector<KOp> build_register_phases(const std::vector<Op> &ops, const int *po
         for (int p = m - 1; p >= 0 && __builtin_popcount(R) < kRpBits; p--) R |= 1u << p;
         KOp k{};
         k.fkind = F_RPHASE;
+        k.nf = layered ? 1 : 0;
         k.k = kRpBits;
         int slot_of[32], tbit_of[32];
         int ns = 0, nt = 0;

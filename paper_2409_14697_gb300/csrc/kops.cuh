@@ -101,12 +101,13 @@ enum RpForm : int { RP_GENERAL = 0, RP_REAL = 1, RP_RX = 2, RP_R0 = 3 };
 // indices for K1, tile-local indices for K2).
 struct KOp {
     int32_t fkind;
-    int32_t nf;         // fixed bits (F_H..F_DENSE2)
+    int32_t nf;         // fixed bits (F_H..F_DENSE2); F_RPHASE: 1 if its pass runs in layers
     int32_t fb[3];      // fixed bits ascending
     int32_t nt;         // touched elements per group; F_CDIAGK: number of non-local terms
     uint64_t set_mask;  // forced-one bits
     uint64_t off[4];    // touched element offsets
-    int32_t k;          // operand count (F_DIAGK / F_DENSEK); F_DENSE1: a D1_* structure class
+    int32_t k;          // operand count (F_DIAGK / F_DENSEK); F_DENSE1: a D1_* structure class;
+                        // F_RPHASE: 1 if the pass may run it in layers
     int32_t pos[8];     // operand positions, first = most significant (F_DIAGK / F_DENSEK)
     int32_t mat;        // offset of the op's reals in the parameter array
     int32_t nmat;       // number of reals

@@ -60,7 +60,7 @@ int launch_pass_ops(DeviceState &st, uint64_t lmask, const std::vector<Op> &fuse
     const int threads = rphase_threads(n, m);
     if (!use_tc && st.dtype == QS_C64 && st.reg_phases && threads) {
         const std::vector<KOp> kp = build_register_phases(fused, pos, m, threads, mats, nullptr,
-                                                           n - m >= kPackTileBits);
+                                                           n - m >= kPackTileBits && has_rotations(fused));
         launch_chunk_pass(st, lmask, kp, mats);
         return (int)kp.size();
     }
@@ -129,6 +129,17 @@ PlanParams plan_params(const DeviceState &st, const qs_options &o) {
         p.sweep_flops = 1e30;  // fuse whenever the block fits: its cost is on the tensor pipe
     }
     return p;
+}
+
+bool has_rotations(const std::vector<Op> &ops) {
+    for (const Op &op : ops)
+        if (op.kind == K_DENSE1 || op.kind == K_CTRL1 || op.kind == K_DENSE) return true;
+    return false;
+}
+
+bool use_register_phases(const std::vector<Op> &ops, int n, const qs_options &o) {
+    if (o.flags & QS_OPT_NO_REG_PHASES) return false;
+    return n < 10 || n >= kTileThreadBits + kRpBits || has_rotations(ops);
 }
 
 PlanParams plan_params(const DeviceState &st, const qs_options &o, const std::vector<Op> &ops) {

@@ -25,6 +25,16 @@ struct Pass {
 PlanParams plan_params(const DeviceState &st, const qs_options &o);
 // The same for a given circuit: the tiles of small complex128 states by its depth.
 PlanParams plan_params(const DeviceState &st, const qs_options &o, const std::vector<Op> &ops);
+// Whether ops hold a matrix besides H and exchanges (circuits and passes of only those and
+// diagonals, as the QFT, are the others).  Those others keep their complex64 arithmetic of one
+// member at a time (of tiles, at 10 to 12 qubits): a transformed random state has <Z> of about
+// 2^(-n/2), whose digits are the states' last bits, and register phases of one tile left it
+// 2.1e-6 off at 11 qubits (tiles: 7e-7).  They would be faster: transform and <Z> at 11 qubits 97
+// us with phases, at 22 qubits 541 us and at 26 qubits 5.6 ms in layers; without, 123 us, 654 us and
+// 8.5 ms.
+bool has_rotations(const std::vector<Op> &ops);
+// DeviceState::reg_phases for a circuit and its options.
+bool use_register_phases(const std::vector<Op> &ops, int n, const qs_options &o);
 // Greedy dependency-respecting partition of ops into passes.
 std::vector<Pass> make_plan(const std::vector<Op> &ops, int n, const PlanParams &pp);
 // The plan QS_MODE_AUTO / CHUNK runs: the greedy plan of ops, or, if it needs fewer passes,
@@ -39,6 +49,7 @@ std::vector<Pass> choose_plan(const std::vector<Op> &ops, int n, const PlanParam
 //     outside the tile stay apart);
 //  3. complex128 FP64 passes of 256 tiles or more: U3 as a real rotation between phases
 //     that join the diagonal runs (smaller states are latency-bound: extra ops cost more);
+//     complex64 register phases in layers (2^kPackTileBits tiles or more): U3 and RX likewise;
 //  4. runs of diagonal gates (a QFT target's controlled phases, the phases of step 3) as
 //     diagonal blocks of up to 8 tile qubits, with factors for qubits outside the tile
 //     (complex64 register phases hold one- and two-qubit diagonals without a sweep).

@@ -364,3 +364,15 @@ def test_rotations_as_shears(qs, n):
     got, _ = _run_c64(qs, n, psi0, gates)
     assert np.max(np.abs(got - want)) <= TOL_C64
     assert fidelity_gap(got, want) <= 1e-6
+
+
+@pytest.mark.parametrize("n", [11, 22])
+def test_transforms_keep_members(qs, n):
+    """Circuits of only H, exchanges and diagonals run neither in phases of one tile nor in layers:
+    the transform of a random state against the oracle."""
+    gates = inputs.qft(n)
+    psi0 = inputs.gaussian_state(n, seed=n).astype(np.complex64)
+    want = oracle.run(psi0.astype(np.complex128), n, gates)
+    got, _ = _run_c64(qs, n, psi0, gates)
+    assert np.max(np.abs(got - want)) <= TOL_C64
+    assert fidelity_gap(got, want) <= 1e-6
