@@ -112,8 +112,9 @@ enum {
                              double: within 0.5 ulp + 2^-56.4 x the largest |matrix entry x
                              amplitude| of the exact value (a chain of FP64 multiply-adds:
                              about one ulp of each partial sum per term).  About one value
-                             in four of every thread runs the native FP64 form, so both
-                             pipes work.  Inputs below 2^-1022 in magnitude count as 0 and
+                             in four (streaming) or eight (chunk passes) of every thread runs
+                             the native FP64 form, so both pipes work.  Inputs below
+                             2^-1022 in magnitude count as 0 and
                              outputs below 2^-959 flush to 0.  Other ops (Hadamards,
                              table-driven diagonal blocks, dense blocks of 2+ qubits) as
                              QS_PREC_FP64. */
@@ -121,8 +122,9 @@ enum {
 
 /* Bits of qs_options.flags (all off by default). */
 enum {
-    QS_OPT_NO_REG_PHASES = 1,   /* complex64 passes over 2^13-amplitude tiles: one shared-memory
-                                   sweep per op instead of register phases (runs of one-qubit,
+    QS_OPT_NO_REG_PHASES = 1,   /* complex64 passes over 2^13-amplitude tiles (states of 10 to 12
+                                   qubits: the one tile they are): one shared-memory sweep per op
+                                   instead of register phases (runs of one-qubit,
                                    controlled and at most two-qubit diagonal gates applied to
                                    amplitudes held in registers, one sweep per run) */
     QS_OPT_NO_DIAG_MERGE = 2,   /* QS_MODE_AUTO / QS_MODE_CHUNK: never merge runs of diagonal
