@@ -629,8 +629,8 @@ __device__ __forceinline__ void rp_store(const float2 (&v)[kRpRegs], float2 *til
 }
 
 // Runs one phase: the 2^nt threads that hold the tile call this.  Bound: instruction issue and
-// fixed latencies (a brickwork pass of 26 qubits issues in 55 % of the cycles, FMA pipe 35 %, shared
-// memory 33 %, HBM 18 %; 4 warps per scheduler, the registers of 32 amplitudes, wait 1.3 of 6
+// fixed latencies (a brickwork pass of 26 qubits issues in 53 % of the cycles, FMA pipe 42 %, shared
+// memory 40 %, HBM 24 %; 4 warps per scheduler, the registers of 32 amplitudes, wait 1.2 of 7
 // cycles per instruction).  So a phase is made of few instructions: a rotation is two shears in
 // place, 32 packed multiply-adds per warp (as a matrix 64; as (1, -t; t, 1) 32 and 32 moves, since
 // both results need both old values: 65.7 ms in the case below), all diagonals between two layers
