@@ -323,8 +323,8 @@ std::vector<Op> split_register_phases(std::vector<Op> ops) {
         r.p0 = a / r.A;
         r.p1 = c / r.S;
         r.q1 = -b / (r.p0 * r.S);
-        const double tol = 1e-14;
-        return std::abs(std::abs(r.q1) - 1.0) <= tol && std::abs(r.p1 * r.q1 * r.A - d) <= tol;
+        const double tol = 1e-14;  // relative to the matrix: QS_DENSE takes any scale
+        return std::abs(std::abs(r.q1) - 1.0) <= tol && std::abs(r.p1 * r.q1 * r.A - d) <= tol * std::max(r.A, r.S);
     };
     int splittable = 0;
     std::vector<char> can(ops.size(), 0);

@@ -261,8 +261,14 @@ struct Packer {
     static bool shears(Matrix &m, bool after, bool may_toggle, bool keep_norm, Term &d, Term &z) {
         if (!m.real) return false;
         const double *u = m.code + 1;
-        const bool reflection = std::fabs(u[0] + u[3]) <= 1e-15 && std::fabs(u[1] - u[2]) <= 1e-15;
-        if (!reflection && (std::fabs(u[0] - u[3]) > 1e-15 || std::fabs(u[1] + u[2]) > 1e-15)) return false;
+        // any matrix may come here (QS_DENSE): equal entries are asked for relative to the largest, and
+        // matrices far from unit scale, whose reals FP32 may not hold to 24 bits, stay as they are
+        double top = 0.0;
+        for (int i = 0; i < 4; i++) top = std::max(top, std::fabs(u[i]));
+        if (!(top >= 0.25 && top <= 4.0)) return false;
+        const double tol = 1e-15 * top;
+        const bool reflection = std::fabs(u[0] + u[3]) <= tol && std::fabs(u[1] - u[2]) <= tol;
+        if (!reflection && (std::fabs(u[0] - u[3]) > tol || std::fabs(u[1] + u[2]) > tol)) return false;
         double a = u[0], b = reflection ? -u[2] : u[2];  // [[a, -b], [b, a]], then a sign if a reflection
         const bool toggle = std::fabs(a) < std::fabs(b);
         if (toggle) {  // X Z after [[b, a], [-a, b]]
