@@ -254,7 +254,8 @@ std::vector<Op> split_one_qubit_phases(const std::vector<Op> &ops) {
         r.s = s;
         r.pf = c / s;
         r.pl = -b / s;
-        const double tol = 1e-14;
+        // relative to the matrix: QS_DENSE takes any scale
+        const double tol = 1e-14 * std::max(std::abs(a), s);
         if (std::abs(r.pl * (-s) - b) > tol || std::abs(r.pf * s - c) > tol ||
             std::abs(r.pf * r.pl * r.a - d) > tol)
             return false;

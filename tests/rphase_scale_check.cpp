@@ -72,6 +72,7 @@ int main(int argc, char **argv) {
                 std::normal_distribution<double> N;
                 for (cd &z : psi) z = cd(N(g), N(g));
                 check(rel_err(run(psi, ops), run(psi, split)) < 1e-12, "split_register_phases", trial);
+                check(rel_err(run(psi, ops), run(psi, split_one_qubit_phases(ops))) < 1e-12, "split_one_qubit_phases", trial);
                 for (const auto *list : {&ops, &split}) {
                     check(packed_error(g, *list, false, trial) < 1e-12, "packed phases", trial);
                     // an account divides at most kMaxDriftFix out, and a rotation's shears take
