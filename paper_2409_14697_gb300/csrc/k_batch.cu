@@ -283,7 +283,7 @@ void batch_build(Batch &b, const std::vector<std::vector<Op>> &circ_ops, const s
             const int threads = rphase_threads(n, m);
             if (!c128 && d.reg_phases && threads) {
                 ko = build_register_phases(fused, pos, m, threads, mt);
-                if (threads < kTileThreadBits) correct_drift(ko, mt);
+                if (threads < kTileThreadBits) correct_drift(ko, mt, d.drift);
             } else {
                 for (const Op &op : fused) ko.push_back(make_kop(op, pos, mt));
             }

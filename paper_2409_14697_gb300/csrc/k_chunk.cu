@@ -322,7 +322,7 @@ void launch_chunk_pass(DeviceState &st, uint64_t lmask, const std::vector<KOp> &
         } else if (phases && a.m < kTileThreadBits + kRpBits) {
             std::vector<KOp> ck = kops;
             std::vector<double> cm = mats;
-            correct_drift(ck, cm);
+            correct_drift(ck, cm, st.drift);
             launch_t<float, false, false>(st, a, ck, cm);
         } else {
             launch_t<float, false, false>(st, a, kops, mats);

@@ -53,8 +53,11 @@ std::vector<KOp> pack_register_phases(const std::vector<KOp> &kops, const std::v
 
 // Register phases as they are (not in layers): one member more at the end of the last, a real
 // factor that takes back what rounding the others' reals to FP32 does to the norm.  For states of
-// one tile, whose gates would otherwise run fused in FP64 and add up less of it.
-void correct_drift(std::vector<KOp> &kops, std::vector<double> &mats);
+// one tile, whose gates would otherwise run fused in FP64 and add up less of it.  What every state
+// suffers alike (equal rotations) is taken back in full; what only equally populated amplitudes
+// do (a phase on some of them) by at most kMaxDriftFix in a call, whose account it is: 3600
+// controlled phases on qubits in |0> change nothing, and an uncapped factor was 3.7e-5 off.
+void correct_drift(std::vector<KOp> &kops, std::vector<double> &mats, RoundingDrift &account);
 
 // Fraction of the state's bytes one streaming application reads and writes, counting
 // whole DRAM sectors of 2^sector_bits elements.

@@ -167,7 +167,7 @@ constexpr int kArenas = 16;
 constexpr int kTpbMaxGroups = 4;
 
 // What rounding matrices and tables to FP32 did to the norm of a state in one call (complex64
-// register phases): logarithms of what is open, and of what tables have been scaled by for it
+// register phases): logarithms of what is open, and of what tables and last members have been scaled by for it
 // (at most kMaxDriftFix in all).
 constexpr double kMaxDriftFix = 6e-6;
 struct RoundingDrift {

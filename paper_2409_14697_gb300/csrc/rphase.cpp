@@ -729,61 +729,99 @@ bool pack_phase(const KOp &ph, const std::vector<double> &in, size_t max_reals, 
     return true;
 }
 
-// Logarithm of the factor by which rounding a diagonal member's reals to FP32 changes the norm, its
-// entries weighted by how many amplitudes take them.
-double diagonal_drift(const double *code) {
+// Logarithm of the factor by which rounding a member's reals to FP32 changes the norm of a state:
+// for every state by at least `sure` (0 where some states gain and others lose), on average over
+// equally populated amplitudes by `mean`.
+struct Change {
+    double sure = 0.0, mean = 0.0;
+};
+
+// of factors that changes lo to hi apply to
+Change between(double lo, double hi, double mean) { return {lo > 0.0 ? lo : hi < 0.0 ? hi : 0.0, mean}; }
+
+Change member_drift(const double *code) {
     const int c = (int)code[0], type = c & 7, J = (c >> 3) & 7, ea = (c >> 6) & 31, eb = (c >> 11) & 31;
     const int len = (c >> 16) & 255;
     const double *P = code + 1;
-    auto change = [&](int i) {  // of the squared modulus of the complex number at P[i]
-        const double r = (double)(float)P[i], m = (double)(float)P[i + 1];
-        const double e = P[i] * P[i] + P[i + 1] * P[i + 1];
-        return e > 0.0 ? (r * r + m * m - e) / e : 0.0;
+    // of squared moduli; what is no rounding (an underflow, an overflow) is not taken back
+    auto change = [](double rounded, double exact) {
+        const double x = exact > 0.0 ? (rounded - exact) / exact : 0.0;
+        return std::fabs(x) <= 1e-6 ? half_log1p(x) : 0.0;
+    };
+    auto square = [](double x) { return x * x; };
+    auto factor = [&](int i) {  // the complex number at P[i]
+        return change(square((float)P[i]) + square((float)P[i + 1]), square(P[i]) + square(P[i + 1]));
+    };
+    // entries at P[first], P[first + step], ...: unweighted, or by binomial weights of n - 1 patterns
+    auto factors = [&](int first, int n, int step, bool binomial) {
+        double lo = factor(first), hi = lo, mean = 0.0, w = binomial ? std::ldexp(1.0, 1 - n) : 1.0 / n;
+        for (int k = 0; k < n; k++) {
+            const double x = factor(first + k * step);
+            lo = std::min(lo, x);
+            hi = std::max(hi, x);
+            mean += w * x;
+            if (binomial) w = w * (n - 1 - k) / (k + 1);
+        }
+        return between(lo, hi, mean);
     };
     switch (type) {
-    case RP_DIAG:
-        return ea == eb ? 0.25 * (change(0) + change(6))
-                        : 0.125 * (change(0) + change(2) + change(4) + change(6));
-    case RP_PARITY: return 0.25 * (change(0) + change(2));
-    case RP_PARITYN: {
-        const int np = (len - 2) / 3;
-        double s = 0.0, w = std::ldexp(1.0, -np);  // binomial weights
-        for (int k = 0; k <= np; k++) {
-            s += w * change(np + 2 * k);
-            w = w * (np - k) / (k + 1);
+    case RP_M1: {
+        cd m[4], r[4];
+        for (int i = 0; i < 4; i++) {
+            const bool off = i == 1 || i == 2;
+            if (eb == RP_REAL) m[i] = P[i];
+            else if (eb == RP_RX) m[i] = off ? cd(0.0, P[i]) : cd(P[i]);
+            else if (eb == RP_R0) m[i] = i ? cd(P[2 * i - 1], P[2 * i]) : cd(P[0]);
+            else m[i] = cd(P[2 * i], P[2 * i + 1]);
+            r[i] = cd((float)m[i].real(), (float)m[i].imag());
         }
-        return 0.5 * s;
+        // squared norms of the columns and how far they are from orthogonal: the squared norm of a
+        // state changes by a factor within x0, x1 and that
+        const double e0 = std::norm(m[0]) + std::norm(m[2]), e1 = std::norm(m[1]) + std::norm(m[3]), e = 0.5 * (e0 + e1);
+        const double was = std::abs(std::conj(m[0]) * m[1] + std::conj(m[2]) * m[3]);
+        if (!(std::fabs(e0 - e1) <= 1e-12 * e && was <= 1e-12 * e)) return {};  // no multiple of a unitary
+        const double x0 = change(std::norm(r[0]) + std::norm(r[2]), e0), x1 = change(std::norm(r[1]) + std::norm(r[3]), e1);
+        const double off = 0.5 * std::abs(std::conj(r[0]) * r[1] + std::conj(r[2]) * r[3]) / e;
+        const double mid = 0.5 * (x0 + x1), spread = std::hypot(0.5 * (x0 - x1), off);
+        return between(mid - spread, mid + spread, mid);
     }
-    case RP_PH: {
-        if (J != 1) return (ea == eb ? 0.25 : 0.125) * change(0);
-        double s = 0.0;
-        for (int q = 0; q < ea; q++) s += 0.25 * change(3 * q + 1);
+    case RP_DIAG: return ea == eb ? factors(0, 2, 6, false) : factors(0, 4, 2, false);
+    case RP_PARITY: return factors(0, 2, 2, false);
+    case RP_PARITYN: return factors((len - 2) / 3, (len - 2) / 3 + 1, 2, true);
+    case RP_PH: {  // amplitudes without the pattern do not change
+        Change s;
+        if (J != 1) s.mean = (ea == eb ? 0.5 : 0.25) * factor(0);
+        for (int q = 0; J == 1 && q < ea; q++) s.mean += 0.5 * factor(3 * q + 1);
         return s;
     }
-    default: return 0.0;
+    default: return {};
     }
 }
 
 }  // namespace
 
-void correct_drift(std::vector<KOp> &kops, std::vector<double> &mats) {
-    double drift = 0.0;
+void correct_drift(std::vector<KOp> &kops, std::vector<double> &mats, RoundingDrift &account) {
+    double sure = 0.0;
     KOp *last = nullptr;
     for (KOp &k : kops) {
         if (k.fkind != F_RPHASE) continue;
         last = &k;
         const double *at = mats.data() + k.mat + 1;
         for (int i = 0; i < (int)mats[(size_t)k.mat]; i++) {
-            const int code = (int)at[0], len = (code >> 16) & 255;
-            drift += rounding_drift(Matrix{at, 1 + len, 0, -1, false, false}) + diagonal_drift(at);
-            at += 1 + len;
+            const Change d = member_drift(at);
+            sure += d.sure;
+            account.open += d.mean - d.sure;
+            at += 1 + (((int)at[0] >> 16) & 255);
         }
     }
+    const double fix = std::min(std::max(account.fixed - account.open, -kMaxDriftFix), kMaxDriftFix) - account.fixed;
     // below an FP32 rounding or so there is nothing to gain; one more member has to fit
-    if (!last || std::fabs(drift) < 1e-7 || last->nmat + 3 > kMaxOpReals) return;
+    if (!last || std::fabs(fix - sure) < 1e-7 || last->nmat + 3 > kMaxOpReals) return;
+    account.fixed += fix;
+    account.open += fix;
     std::vector<double> prog(mats.begin() + last->mat, mats.begin() + last->mat + last->nmat);
     prog[0] += 1.0;
-    prog.insert(prog.end(), {(double)(RP_PH | kRpAlways << 6 | kRpAlways << 11 | 2 << 16), std::exp(-drift), 0.0});
+    prog.insert(prog.end(), {(double)(RP_PH | kRpAlways << 6 | kRpAlways << 11 | 2 << 16), std::exp(fix - sure), 0.0});
     last->mat = (int32_t)mats.size();
     last->nmat = (int32_t)prog.size();
     mats.insert(mats.end(), prog.begin(), prog.end());
