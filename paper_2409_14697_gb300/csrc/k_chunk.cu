@@ -314,7 +314,8 @@ void launch_chunk_pass(DeviceState &st, uint64_t lmask, const std::vector<KOp> &
             layers |= k.fkind == F_RPHASE && k.nf;
         }
         const size_t taken = (B << a.m) + kops.size() * sizeof(KOp);
-        const size_t limit = staged_limit<float, false, false, true>();
+        // (staged_limit loads the kernel it asks about: not for passes that run another)
+        const size_t limit = layers ? staged_limit<float, false, false, true>() : 0;
         if (layers && n - a.m >= kPackTileBits && taken < limit) {
             std::vector<double> packed;
             const std::vector<KOp> pk = pack_register_phases(kops, mats, (limit - taken) / sizeof(float), packed, &st.drift);
@@ -329,5 +330,7 @@ void launch_chunk_pass(DeviceState &st, uint64_t lmask, const std::vector<KOp> &
         }
     }
 }
+
+const void *chunk_kernel() { return (const void *)k_chunk<float, false, false, false>; }
 
 }  // namespace qs

@@ -395,4 +395,6 @@ void build_tc_operand(const std::vector<cd> &G, int k, std::vector<float> &out, 
     count = (int)(2 * nf);
 }
 
+const void *fused_tc_kernel() { return (const void *)k_chunk_tc; }
+
 }  // namespace qs

@@ -200,4 +200,6 @@ void launch_phasefn(DeviceState &st, const Op &op) {
     else launch_t<float, false>(st, *op.pf);
 }
 
+const void *phasefn_kernel() { return (const void *)k_phasefn<float, false>; }
+
 }  // namespace qs

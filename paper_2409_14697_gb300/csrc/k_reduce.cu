@@ -1078,6 +1078,8 @@ void topk_launch(DeviceState &st, uint32_t K, uint64_t *idx_dev, double *amp_dev
 
 }  // namespace
 
+const void *reduce_kernel() { return (const void *)k_set_one; }
+
 void top_k_async(DeviceState &st, uint32_t K, uint64_t *idx_dev, double *amp_dev) {
     topk_launch(st, K, idx_dev, amp_dev, TopkSelect::all);
 }

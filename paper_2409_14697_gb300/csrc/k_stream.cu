@@ -749,4 +749,6 @@ void launch_stream_op(DeviceState &st, const Op &op) {
     else launch_typed<float>(st, op);
 }
 
+const void *stream_kernel() { return (const void *)k_diag_general<double, 1>; }
+
 }  // namespace qs

@@ -131,4 +131,6 @@ void launch_tpb_product(DeviceState &st, const void *const *tables, const uint64
     count_launch();
 }
 
+const void *tpb_kernel() { return (const void *)k_tpb<float, 2>; }
+
 }  // namespace qs

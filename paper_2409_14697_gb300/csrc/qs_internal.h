@@ -247,6 +247,14 @@ void launch_scale_ratio(DeviceState &st, const double *norms_dev);
 void top_k_async(DeviceState &st, uint32_t k, uint64_t *idx_dev, double *amp_dev);
 size_t scratch_expz_bytes(int n);
 size_t scratch_topk_bytes(int n, uint32_t k);
+// A kernel of each file whose kernels a request of the server may launch.  The kernels of a file
+// are one library to the driver, which server.cpp loads whole.
+const void *stream_kernel();
+const void *chunk_kernel();
+const void *phasefn_kernel();
+const void *fused_tc_kernel();
+const void *tpb_kernel();
+const void *reduce_kernel();
 
 // Host <-> device copy of `bytes` on st.stream (asynchronous).  Ranges of page-locked host
 // memory mapped into the device (cudaHostAlloc, registered memory) of 4 MiB or more are

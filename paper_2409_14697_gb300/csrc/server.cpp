@@ -22,6 +22,8 @@
 #include <unordered_map>
 #include <unordered_set>
 
+#include <cuda.h>
+
 #include "capi_util.h"
 #include "qs_internal.h"
 
@@ -137,6 +139,44 @@ void presize_slot(Slot &s, int n, uint32_t k) {
     ensure_scratch(d, std::max(scratch_expz_bytes(n), scratch_topk_bytes(n, kk)));
     presize_results(s);
     arena_reserve(d, (size_t)1 << 20);
+}
+
+// Loads every kernel of the library that holds `entry`.  The driver loads a kernel at its first
+// launch, and what is launched from then on waits for the work in flight: the small requests of a
+// process's first stream of 120 (2000 per second) stood behind its first large one, 0.39-0.66 s at the
+// median, and 0.07-0.35 s in its second stream; with all kernels loaded both take 0.07-0.26 s (what is
+// left is the link's share, which differs from process to process).  203 kernels take about as long
+// as creating the context does without them.  Where the driver cannot list a library, its kernels
+// load as they are used.
+void load_kernels(const void *entry) {
+    auto driver = [](const char *name, unsigned version, auto &fn) {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion(name, &p, version, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess)
+            p = nullptr;
+        fn = (std::remove_reference_t<decltype(fn)>)p;
+        return p != nullptr;
+    };
+    CUresult (*library_of)(CUlibrary *, CUkernel) = nullptr;
+    CUresult (*count_of)(unsigned *, CUlibrary) = nullptr;
+    CUresult (*list)(CUkernel *, unsigned, CUlibrary) = nullptr;
+    CUresult (*function_of)(CUfunction *, CUkernel) = nullptr;
+    CUresult (*load)(CUfunction) = nullptr;
+    cudaKernel_t kernel = nullptr;
+    CUlibrary lib = nullptr;
+    unsigned n = 0;
+    if (driver("cuKernelGetLibrary", 12050, library_of) && driver("cuLibraryGetKernelCount", 12040, count_of) &&
+        driver("cuLibraryEnumerateKernels", 12040, list) && driver("cuKernelGetFunction", 12000, function_of) &&
+        driver("cuFuncLoad", 12040, load) && cudaGetKernel(&kernel, entry) == cudaSuccess &&
+        library_of(&lib, (CUkernel)kernel) == CUDA_SUCCESS && count_of(&n, lib) == CUDA_SUCCESS) {
+        std::vector<CUkernel> kernels(n);
+        CUfunction f = nullptr;
+        if (list(kernels.data(), n, lib) == CUDA_SUCCESS)
+            for (CUkernel k : kernels)
+                if (function_of(&f, k) == CUDA_SUCCESS) load(f);
+    }
+    cudaGetLastError();  // not an error: clear it so later launch checks do not see it
 }
 
 }  // namespace
@@ -343,6 +383,10 @@ int qs_server_create(const qs_server_config *cfg, qs_server **out) {
     S.cfg = *cfg;
     try {
         QS_CUDA(cudaGetDevice(&S.device));
+        QS_CUDA(cudaFree(nullptr));  // kernels are loaded into a context: there has to be one
+        for (const void *entry : {stream_kernel(), chunk_kernel(), phasefn_kernel(), fused_tc_kernel(), tpb_kernel(),
+                                  reduce_kernel()})
+            load_kernels(entry);
         // a pool of the server's own for the request states: freed state memory stays in it for
         // reuse, but an allocation never reuses memory whose free is still pending on another
         // slot's stream (that would make the new request wait for the old one's work)
