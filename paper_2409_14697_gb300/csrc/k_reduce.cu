@@ -69,12 +69,14 @@ struct SumF64 {
 };
 // Sums of squares as integers.  E: the biased exponent of the group's largest |x|.  A real x of
 // the group becomes X = floor(|x| 2^(1083 - E)) < 2^61 (its significand shifted right by E - e),
-// its square the top 64 bits of X^2, short of the exact value by less than 6 units of
-// 2^(2 E - 2102) (3 from the shifted X, 3 from the low words), 2^-56 of the largest square at most 6
-// times.  A group's sum of up to 32 squares is below 2^63 and exact beyond that, so it is
-// within 32 * 6 units of its exact value, 2^-50.4 of its largest square and, as the units lost
-// are those of the many terms that make the sum large, about 2^-54 of a sum of comparable
-// terms: the rounding of a FP64 chain.  One integer-to-double conversion per group sum.
+// its square the top 64 bits of X^2 in units of 2^(2 E - 2102): at least 2^56 units for the largest
+// real.  A square falls short by less than 1.125 units (X by less than 1 of at most 2^60 where bits
+// were shifted out, the product by less than 1) and is over by at most 0.25 (from the square of the
+// low word, which xl stands for).  A group's sum of up to 32 squares is below 2^63 and exact beyond
+// that: within 36 units, 2^-50.8 of its largest square, which a group of one large real and 31
+// middling ones comes near; of a sum of comparable terms about 2^-56, less than the rounding of an
+// FP64 chain.  (2 mulhi(xh, xl) in the second term lost up to 3.25 units a square, such a group
+// 2^-49.3.)  One integer-to-double conversion per group sum.
 // 20 integer instructions per real against 1.25-1.75 FP64 instructions (16 times slower each).
 struct SumU64 {
     using T = unsigned long long;
@@ -88,7 +90,8 @@ struct SumU64 {
         unsigned long long X = ((unsigned long long)__funnelshift_l(lo, mh, 8) << 32) | (lo << 8);
         asm("shr.b64 %0, %0, %1;" : "+l"(X) : "r"(E - e));
         const uint32_t xh = (uint32_t)(X >> 32), xl = (uint32_t)X;
-        return (unsigned long long)xh * xh + 2ull * __umulhi(xh, xl);
+        // xl stands for xl^2 / 2^32, from which it differs by at most 2^30 (a quarter unit)
+        return (unsigned long long)xh * xh + __umulhi(2u * xh + 1u, xl);
     }
     static __device__ __forceinline__ T leaf(double2 a, uint32_t E) { return square(a.x, E) + square(a.y, E); }
     static __device__ __forceinline__ double to_double(T a, uint32_t E) {
