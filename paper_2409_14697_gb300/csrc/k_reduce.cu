@@ -629,7 +629,9 @@ struct TkState {
     int done;                // 1: the sampled selection is complete
 };
 
-// Sample of one line of 128 bytes in every 2^sb: element of sample slot i.
+// Sample of one line of 128 bytes in every 2^sb: element of sample slot i.  The multipliers are
+// published hash constants: 2^32 over the golden ratio and a second prime, as xxHash has them, and one
+// of C. Wellons's search for low-bias 32-bit hashes.
 template <typename V>
 __device__ __forceinline__ uint64_t sample_index(uint64_t i, int sb) {
     constexpr int LB = sizeof(V) == 16 ? 3 : 4;  // elements per line

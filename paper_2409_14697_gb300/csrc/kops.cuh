@@ -107,7 +107,7 @@ struct KOp {
     uint64_t set_mask;  // forced-one bits
     uint64_t off[4];    // touched element offsets
     int32_t k;          // operand count (F_DIAGK / F_DENSEK); F_DENSE1: a D1_* structure class;
-                        // F_RPHASE: 1 if the pass may run it in layers
+                        // F_RPHASE: kRpBits
     int32_t pos[8];     // operand positions, first = most significant (F_DIAGK / F_DENSEK)
     int32_t mat;        // offset of the op's reals in the parameter array
     int32_t nmat;       // number of reals
