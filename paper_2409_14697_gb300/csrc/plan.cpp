@@ -139,7 +139,17 @@ bool has_rotations(const std::vector<Op> &ops) {
 
 bool use_register_phases(const std::vector<Op> &ops, int n, const qs_options &o) {
     if (o.flags & QS_OPT_NO_REG_PHASES) return false;
-    return n < 10 || n >= kTileThreadBits + kRpBits || has_rotations(ops);
+    if (n < 10 || n >= kTileThreadBits + kRpBits) return true;
+    if (!has_rotations(ops)) return false;
+    if (n > 10) return true;
+    // 10 qubits: a phase is one warp's, and exchanges and wide blocks between gates that phases hold
+    // cut them short.  One in 48 and more of those: tiles (random gates of all types, 6 % exchanges:
+    // 150 of them 124 us in tiles, 131 in phases; 300 in a batch of 64 136 and 158); fewer: phases
+    // (without exchanges 118 us in phases, 133 in tiles).  11 qubits: phases win with them too.  Blocks
+    // for the most part make no phases either way.
+    size_t others = 0;
+    for (const Op &op : ops) others += op.kind == K_SWAP || op.kind == K_DENSE;
+    return 48 * others < ops.size() || 4 * others >= 3 * ops.size();
 }
 
 PlanParams plan_params(const DeviceState &st, const qs_options &o, const std::vector<Op> &ops) {
