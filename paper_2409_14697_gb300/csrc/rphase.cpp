@@ -30,9 +30,11 @@
 // The device's reals are FP32, and the rounding of an angle that a circuit repeats (Trotter
 // steps) changes the norm the same way each time.  What the matrices and the tables so far have
 // changed it by is divided out of the next table, whose own rounding then joins the account
-// (RoundingDrift): the 25-qubit Trotter circuit of 16 steps ended up to 1.1e-5 off, now 5e-7.
-// A call never divides out more than kMaxDriftFix, so that its result also stays as near to what
-// the plain FP32 matrices of the other execution modes give.
+// (RoundingDrift).  The 25-qubit Trotter circuit of 16 steps and its <Z> were 1.8e-5 to 2.3e-5 off
+// with members alone, now 6.0e-6 to 8.5e-6 (four seeds); one of 23 qubits and 4 steps 4.3e-6, now
+// 6.9e-7.  The account takes amplitudes as equally populated.  A call never divides out more than
+// kMaxDriftFix, so that a state that is not (thousands of phases on qubits in |0>) is no further off than
+// that, and the result stays near to what the plain FP32 matrices of the other execution modes give.
 #include <algorithm>
 #include <cmath>
 

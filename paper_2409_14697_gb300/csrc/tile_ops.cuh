@@ -636,8 +636,9 @@ __device__ __forceinline__ void rp_store(const float2 (&v)[kRpRegs], float2 *til
 // both results need both old values: 65.7 ms in the case below), all diagonals between two layers
 // of rotations one complex multiply and half a load per amplitude, one read of the program per
 // layer.  28-qubit brickwork of 40 layers 117.5 ms with members alone, 74.4 in layers, 66.8 with
-// offsets in bytes and run offsets made once, 56.3 with shears; 30-qubit QAOA p = 4 99.6, 71.6 and,
-// with shears, 69.4 ms; 25-qubit Trotter circuit of 16 steps 7.4, 4.94, 4.42 ms.  LAYERS: the program is in layers
+// offsets in bytes and run offsets made once, 56.3 with shears; 25-qubit Trotter circuit of 16 steps
+// 7.4, 4.94, 4.42 ms; 30-qubit QAOA p = 4, whose time differs from machine to machine, 96 to 67, 108 to
+// 75 and 125 to 86 ms from members alone to shears.  LAYERS: the program is in layers
 // (passes of many tiles); else it is a member count and the members.  Two instances, since
 // reading both in one cost the plain form 12 % (small states wait for single tiles).
 template <bool LAYERS>
